@@ -15,6 +15,7 @@
 
 #include "ff.h"
 #include "ff_kernels.cuh"
+#include "ff_seed_tc.cuh"
 
 using namespace ffk;
 
@@ -116,14 +117,11 @@ __global__ void k_dense(const uint8_t *__restrict__ feat, int N, int8_t *__restr
 }
 
 // ---------------------------------------------------------------------------
-// seeding: exact top-8 by (squared distance, linear index) of level-0 WHT
-// vectors (Sec. 3.1 Eq. 1, Sec. 3.2 Eq. 4; kd-tree leaf replaced by the exact
-// nearest neighbours it approximates)
+// the allocation-free seeding search (ff_seed_knn_static): exact top-8 by
+// (squared distance, linear index) of level-0 WHT vectors (Sec. 3.1 Eq. 1,
+// Sec. 3.2 Eq. 4; kd-tree leaf replaced by the exact nearest neighbours it
+// approximates); the contexts' own search is in ff_seed_tc.cuh
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool lex_less(int d, int i, int D, int I) {
-    return d < D || (d == D && i < I);
-}
-
 // insert (d, i) into the ascending list (D, I) of 8, dropping the last entry
 __device__ __forceinline__ void list_insert(int (&D)[8], int (&I)[8], int d, int i) {
 #pragma unroll
@@ -258,37 +256,6 @@ __global__ void k_seed_merge(const int2 *__restrict__ part, int nchunks, int NQ,
     }
 }
 
-// Phase 3 (Eq. 1 rerank): each candidate p2 gives F = 8 (p2 - p); keep the
-// lowest E at the coarsest scale, the earlier rank on ties.
-template <int C>
-__global__ void k_seed_rerank(const int *__restrict__ knn_idx, int leaf, const uint8_t *f1L,
-                              const uint8_t *f2L, int W, int H, int L, int WL, int HL,
-                              uint32_t *__restrict__ flow, int *__restrict__ cost) {
-    constexpr int P = Geo<C>::P;
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= WL * HL) return;
-    const int gy = q / WL, gx = q - gy * WL;
-    const int px = gx << L, py = gy << L;
-    uint32_t qw[P / 4];
-#pragma unroll
-    for (int w = 0; w < P / 4; w++) qw[w] = ldg32(f1L + (size_t)q * P + 4 * w);
-    uint32_t bf = kFlowInvalid;
-    int bc = kCostInvalid;
-    for (int r = 0; r < leaf; r++) {
-        const int idx = knn_idx[(size_t)q * leaf + r];
-        if (idx < 0) break;
-        int fx = 8 * (idx % W - px), fy = 8 * (idx / W - py);
-        clamp_flow(W, H, px, py, fx, fy);
-        const int e = sad_full<C>(f2L, make_tap<P>(px, py, fx, fy, L, WL, HL), qw);
-        if (e < bc) {
-            bc = e;
-            bf = pack_flow(fx, fy);
-        }
-    }
-    flow[q] = bf;
-    cost[q] = bc;
-}
-
 // caller-supplied seeds on the coarsest grid: clamp and evaluate
 template <int C>
 __global__ void k_seed_given(const uint32_t *__restrict__ seeds, const uint8_t *f1L,
@@ -342,9 +309,7 @@ __global__ void k_upsample(const uint32_t *__restrict__ pflow, int WP, const uin
 
 #include "ff_sweep.cuh"
 #include "ff_peaks.cuh"
-#include "ff_seed.cuh"
 #include "ff_wht_tc.cuh"
-#include "ff_seed_tc.cuh"
 
 // ---- region filter (Sec. 3.7) ------------------------------------------
 // Kept points are joined into regions by a lock-free union-find: a root only
@@ -541,7 +506,6 @@ constexpr int kNumDirs = 3;   // forward, backward, second backward
 constexpr int kMaxChunks = 64;
 constexpr int kCtasPerSm = 8;     // seeding grids: about this many CTAs per SM
 constexpr int kSeedQpt = 2;
-constexpr int kSeedSample = 16;   // candidate subsampling of the bound pass
 constexpr int kSeedQueriesPerCta = 128 * kSeedQpt;
 
 struct DirState {
@@ -549,14 +513,8 @@ struct DirState {
     int *cost[2] = {nullptr, nullptr};
     unsigned long long *edge = nullptr;
     unsigned int *ticket = nullptr;           // [FF_MAX_SCALES * kMaxIters]
-    int *knn_idx = nullptr;
-    int *knn_dist = nullptr;
-    int2 *part = nullptr;                     // seeding scratch: per-chunk lists
-    __nv_bfloat16 *qbf = nullptr;             // seeding queries, bf16 rows of K
-    int *qnorm = nullptr;                     //   their squared norms
-    float *t0 = nullptr;                      //   upper bounds of their 8th key
-    __nv_bfloat16 *cbf = nullptr;             // seeding candidates, bf16 rows of K
-    uint8_t *qtile = nullptr, *ctile = nullptr;   // the same in 128-row tensor-core tiles
+    uint8_t *qtile = nullptr, *ctile = nullptr;   // seeding: 128-row tensor-core tiles
+    uint32_t *lists = nullptr;                //   and each query's lists of tiles
     int *err = nullptr;
 };
 
@@ -587,7 +545,6 @@ struct ff_ctx {
     uint8_t *rf_flag = nullptr;
     unsigned long long wait_ns = 2000000000ull;
     int sweep_lanes = 4;   // propagation-warp lanes per grid point in the sweep: 2, 4 or 8
-    int seed_tc = 1;       // seeding full pass on tcgen05 (0: mma.sync)
     int force_timeout = 0;
     long long launches = 0;
     std::string last_error;
@@ -764,15 +721,9 @@ void free_all(ff_ctx *c) {
         cudaFree(d.cost[1]);
         cudaFree(d.edge);
         cudaFree(d.ticket);
-        cudaFree(d.knn_idx);
-        cudaFree(d.knn_dist);
-        cudaFree(d.part);
-        cudaFree(d.qbf);
-        cudaFree(d.qnorm);
-        cudaFree(d.t0);
-        cudaFree(d.cbf);
         cudaFree(d.qtile);
         cudaFree(d.ctile);
+        cudaFree(d.lists);
         cudaFree(d.err);
     }
     cudaFree(c->pair_mask);
@@ -824,125 +775,67 @@ void seed_geometry(int nq, int ncand, int sms, int *nchunks, int *chunk) {
     *nchunks = (ncand + ch - 1) / ch;
 }
 
-// seeding geometry of the mma.sync scan: 64 queries per CTA, candidates
-// split into chunks (whole 64-candidate tiles) so the grid holds about four
-// CTAs per SM of the device (sms): long chunks, few restarts
-void seed_geometry_mma(int nq, int ncand, int sms, int *nchunks, int *chunk) {
-    const int qt = (nq + 63) / 64;
-    int nc = (4 * sms + qt - 1) / qt;
-    nc = nc < 1 ? 1 : (nc > kMaxChunks ? kMaxChunks : nc);
-    int ch = (ncand + nc - 1) / nc;
-    ch = ((ch + 63) / 64) * 64;
-    if (ch < 512) ch = 512;
-    *chunk = ch;
-    *nchunks = (ncand + ch - 1) / ch;
+// How the seeding's product is split: nqt tiles of 128 queries by nch chunks of
+// `chunk` tiles of 128 candidates.  Two CTAs share an SM, so `slots` run at
+// once; among the chunk counts the one whose waves take the fewest tiles is
+// taken, a CTA's start counting as kTcStartTiles.  (One wave of 5 chunks at
+// 1024x436 leaves 29 of 304 slots idle, two waves of 11 leave 3.)
+constexpr int kTcStartTiles = 24, kTcMaxChunks = 16, kTcMaxSlots = 512;
+struct SeedSplit {
+    int nqt, nct, nch, chunk;
+};
+SeedSplit seed_split(size_t nq, size_t ncand, int slots) {
+    SeedSplit z;
+    z.nqt = (int)((nq + kTcRows - 1) / kTcRows);
+    z.nct = (int)((ncand + kTcRows - 1) / kTcRows);
+    const int least = (z.nct + kTcChunkTiles - 1) / kTcChunkTiles;
+    // few queries: chunks enough for one wave
+    const int most = max(least, min(z.nct, max(kTcMaxChunks, slots / z.nqt)));
+    long long best = 0;
+    z.nch = 0;
+    for (int n = least; n <= most; n++) {
+        const long long waves = ((long long)z.nqt * n + slots - 1) / slots;
+        const long long t = waves * ((z.nct + n - 1) / n + kTcStartTiles);
+        if (z.nch == 0 || t < best) best = t, z.nch = n;
+    }
+    z.chunk = (z.nct + z.nch - 1) / z.nch;
+    z.nch = (z.nct + z.chunk - 1) / z.chunk;
+    return z;
+}
+// list entries that hold every frame of up to ncand candidates and nq queries
+size_t seed_list_words(size_t nq, size_t ncand) {
+    const size_t nqt = (nq + kTcRows - 1) / kTcRows, nct = (ncand + kTcRows - 1) / kTcRows;
+    const size_t least = (nct + kTcChunkTiles - 1) / kTcChunkTiles;
+    const size_t most = max(least, (size_t)kTcMaxChunks);
+    return kTcRows * 8 * max(nqt * most, (size_t)kTcMaxSlots);
 }
 
-ff_status launch_seed_knn(ff_ctx *c, int d, const uint8_t *fs, const uint8_t *fd, int W, int H) {
+// The seeding search of one direction (ff_seed_tc.cuh): the queries are the
+// coarsest grid's points, and each query's result goes where `out` says.
+template <int C>
+ff_status launch_seed(ff_ctx *c, int d, const uint8_t *fs, const uint8_t *fd, int W, int H,
+                      const KnnOut &out) {
+    constexpr int KS = C == 1 ? 1 : 2;
     DirState &st = c->dir[d];
-    const int S = c->S, N = 1 << (S - 1);
     int WS, HS;
-    level_dims(W, H, S - 1, &WS, &HS);
-    const int nq = WS * HS;
+    level_dims(W, H, c->S - 1, &WS, &HS);
+    const int nq = WS * HS, N = 1 << (c->S - 1);
     const int stride = c->cfg.seed_stride;
     const int Wc = (W + stride - 1) / stride, Hc = (H + stride - 1) / stride;
     const int ncand = Wc * Hc;
-    // bf16 rows of the queries (coarsest grid) and candidates (stride grid)
+    const SeedSplit z = seed_split(nq, ncand, min(2 * c->sms, kTcMaxSlots));
+    ff_status s;
     prof_begin(c, "k_seed_prep");
-    if (c->C == 1)
-        k_seed_prep<1, 16, true><<<(nq + 127) / 128, 128, 0, c->stream>>>(fs, W, N, WS, HS, st.qbf,
-                                                                         st.qnorm);
-    else
-        k_seed_prep<3, 32, true><<<(nq + 127) / 128, 128, 0, c->stream>>>(fs, W, N, WS, HS, st.qbf,
-                                                                         st.qnorm);
-    ff_status s = check_launch(c, "k_seed_prep");
-    if (s) return s;
-    prof_begin(c, "k_seed_prep");
-    if (c->C == 1)
-        k_seed_prep<1, 16, false><<<(ncand + 127) / 128, 128, 0, c->stream>>>(
-            fd, W, stride, Wc, Hc, st.cbf, nullptr);
-    else
-        k_seed_prep<3, 32, false><<<(ncand + 127) / 128, 128, 0, c->stream>>>(
-            fd, W, stride, Wc, Hc, st.cbf, nullptr);
-    s = check_launch(c, "k_seed_prep");
-    if (s) return s;
-    // bound pass over every kSeedSample-th candidate: the 8th key of each
-    // chunk of the sample bounds the query's final 8th key from above
-    const int ns = (ncand + kSeedSample - 1) / kSeedSample;
-    int nchunks1, chunk1;
-    seed_geometry_mma(nq, ns, c->sms, &nchunks1, &chunk1);
-    {
-        dim3 grid1((nq + 63) / 64, nchunks1);
-        prof_begin(c, "k_seed_scan");
-        if (c->C == 1)
-            k_seed_mma<1><<<grid1, 128, 0, c->stream>>>(st.qbf, st.qnorm, st.cbf, nq, ns, chunk1,
-                                                        kSeedSample, W, stride, Wc, nullptr, 0,
-                                                        st.t0, st.part);
-        else
-            k_seed_mma<2><<<grid1, 128, 0, c->stream>>>(st.qbf, st.qnorm, st.cbf, nq, ns, chunk1,
-                                                        kSeedSample, W, stride, Wc, nullptr, 0,
-                                                        st.t0, st.part);
-        s = check_launch(c, "k_seed_scan");
-        if (s) return s;
-    }
-    int nchunks, chunk;
-    if (c->seed_tc) {
-        // full pass on tcgen05: 128-row tiles of queries and candidates
-        const int K = c->C == 1 ? 16 : 32, DH2 = 9 * c->C;
-        const int nq_t = (nq + kTcRows - 1) / kTcRows;
-        const int nc_pad = (ncand + kTcRows - 1) / kTcRows * kTcRows;
-        prof_begin(c, "k_seed_prep");
-        if (K == 16) {
-            k_seed_tile<16><<<(nq_t * kTcRows * 2 + 255) / 256, 256, 0, c->stream>>>(st.qbf, nq, -1,
-                                                                                 st.qtile);
-        } else {
-            k_seed_tile<32><<<(nq_t * kTcRows * 4 + 255) / 256, 256, 0, c->stream>>>(st.qbf, nq, -1,
-                                                                                 st.qtile);
-        }
-        if ((s = check_launch(c, "k_seed_prep"))) return s;
-        prof_begin(c, "k_seed_prep");
-        if (K == 16)
-            k_seed_tile<16><<<(nc_pad * 2 + 255) / 256, 256, 0, c->stream>>>(st.cbf, ncand, DH2,
-                                                                          st.ctile);
-        else
-            k_seed_tile<32><<<(nc_pad * 4 + 255) / 256, 256, 0, c->stream>>>(st.cbf, ncand, DH2,
-                                                                          st.ctile);
-        if ((s = check_launch(c, "k_seed_prep"))) return s;
-        // one wave of two CTAs per SM (tensor memory holds two): split the
-        // candidates into 128-aligned chunks
-        int nc = (2 * c->sms) / nq_t;
-        nc = nc < 1 ? 1 : (nc > kMaxChunks / 2 ? kMaxChunks / 2 : nc);
-        chunk = (ncand + nc - 1) / nc;
-        chunk = (chunk + kTcRows - 1) / kTcRows * kTcRows;
-        nchunks = (ncand + chunk - 1) / chunk;
-        prof_begin(c, "k_seed_scan");
-        if (c->C == 1)
-            k_seed_tc<1><<<dim3(nq_t, nchunks), 320, tc_seed_smem_bytes<1>(), c->stream>>>(
-                st.qtile, st.qnorm, st.ctile, nq, ncand, chunk, W, stride, Wc, st.t0, nchunks1,
-                st.part, st.err, c->wait_ns);
-        else
-            k_seed_tc<2><<<dim3(nq_t, nchunks), 320, tc_seed_smem_bytes<2>(), c->stream>>>(
-                st.qtile, st.qnorm, st.ctile, nq, ncand, chunk, W, stride, Wc, st.t0, nchunks1,
-                st.part, st.err, c->wait_ns);
-        if ((s = check_launch(c, "k_seed_scan"))) return s;
-        nchunks *= 2;   // two lists per chunk
-    } else {
-        seed_geometry_mma(nq, ncand, c->sms, &nchunks, &chunk);
-        dim3 grid((nq + 63) / 64, nchunks);
-        prof_begin(c, "k_seed_scan");
-        if (c->C == 1)
-            k_seed_mma<1><<<grid, 128, 0, c->stream>>>(st.qbf, st.qnorm, st.cbf, nq, ncand, chunk,
-                                                       1, W, stride, Wc, st.t0, nchunks1, nullptr,
-                                                       st.part);
-        else
-            k_seed_mma<2><<<grid, 128, 0, c->stream>>>(st.qbf, st.qnorm, st.cbf, nq, ncand, chunk,
-                                                       1, W, stride, Wc, st.t0, nchunks1, nullptr,
-                                                       st.part);
-        if ((s = check_launch(c, "k_seed_scan"))) return s;
-    }
+    k_seed_prep<C><<<z.nct + z.nqt, kTcRows, 0, c->stream>>>(fs, fd, W, N, WS, nq, stride, Wc,
+                                                             ncand, st.qtile, st.ctile);
+    if ((s = check_launch(c, "k_seed_prep"))) return s;
+    prof_begin(c, "k_seed_scan");
+    k_seed_tc<KS><<<dim3(z.nqt, z.nch), 192, tc_seed_smem_bytes<KS>(), c->stream>>>(
+        st.qtile, st.ctile, z.nct, z.chunk, st.lists, st.err, c->wait_ns);
+    if ((s = check_launch(c, "k_seed_scan"))) return s;
     prof_begin(c, "k_seed_merge");
-    k_seed_merge<<<(nq + 127) / 128, 128, 0, c->stream>>>(st.part, nchunks, nq, c->cfg.seed_leaf,
-                                                         st.knn_idx, st.knn_dist);
+    k_seed_pick<C><<<(nq + 3) / 4, 128, 0, c->stream>>>(fs, fd, W, N, WS, nq, stride, Wc, ncand,
+                                                        st.lists, z.nqt, z.nch, z.chunk, out);
     return check_launch(c, "k_seed_merge");
 }
 
@@ -1023,15 +916,6 @@ ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L,
 }
 
 template <int C>
-void launch_rerank(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L, int W, int H, int L,
-                   int WL, int HL, uint32_t *flow, int *cost) {
-    const int nq = WL * HL;
-    prof_begin(c, "k_seed_rerank");
-    k_seed_rerank<C><<<(nq + 127) / 128, 128, 0, c->stream>>>(
-        c->dir[d].knn_idx, c->cfg.seed_leaf, f1L, f2L, W, H, L, WL, HL, flow, cost);
-}
-
-template <int C>
 void launch_given(ff_ctx *c, const uint32_t *seeds, const uint8_t *f1L, const uint8_t *f2L, int W,
                   int H, int L, int WL, int HL, uint32_t *flow, int *cost) {
     const int nq = WL * HL;
@@ -1101,13 +985,10 @@ ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seed
                                     cost);
                 s = check_launch(c, "k_seed_given");
             } else {
-                s = launch_seed_knn(c, d, fsrc, fdst, W, H);
-                if (s) return s;
-                if (c->C == 1)
-                    launch_rerank<1>(c, d, f1L, f2L, W, H, L, WL, HL, flow, cost);
-                else
-                    launch_rerank<3>(c, d, f1L, f2L, W, H, L, WL, HL, flow, cost);
-                s = check_launch(c, "k_seed_rerank");
+                const KnnOut out{c->cfg.seed_leaf, nullptr, nullptr, f1L, f2L, W, H, L,
+                                 WL, HL, flow, cost};
+                s = c->C == 1 ? launch_seed<1>(c, d, fsrc, fdst, W, H, out)
+                              : launch_seed<3>(c, d, fsrc, fdst, W, H, out);
             }
         } else {
             if (c->C == 1)
@@ -1369,7 +1250,7 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return FF_ECUDA;
     DeviceGuard guard(device);
-    // the tensor-core seeding kernel takes more than 48 KB of shared memory
+    // the seeding's candidate ring takes more than 48 KB of shared memory
     if (cudaFuncSetAttribute(k_seed_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc_seed_smem_bytes<1>()) != cudaSuccess ||
         cudaFuncSetAttribute(k_seed_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1416,17 +1297,10 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
         if (e == cudaSuccess) e = alloc(&d.edge, c->edge_cap);
         if (e == cudaSuccess) e = cudaMemset(d.edge, 0, c->edge_cap * sizeof(unsigned long long));
         if (e == cudaSuccess) e = alloc(&d.ticket, (size_t)FF_MAX_SCALES * kMaxIters);
-        if (e == cudaSuccess) e = alloc(&d.knn_idx, c->nq_cap * FF_MAX_LEAF);
-        if (e == cudaSuccess) e = alloc(&d.knn_dist, c->nq_cap * FF_MAX_LEAF);
-        if (e == cudaSuccess) e = alloc(&d.part, c->nq_cap * kMaxChunks * 8);
-        const size_t K = c->C == 1 ? 16 : 32;
-        if (e == cudaSuccess) e = alloc(&d.qbf, c->nq_cap * K);
-        if (e == cudaSuccess) e = alloc(&d.qnorm, c->nq_cap);
-        if (e == cudaSuccess) e = alloc(&d.t0, c->nq_cap * kMaxChunks);
-        if (e == cudaSuccess) e = alloc(&d.cbf, npix * K);
-        const size_t pad = kTcRows;
+        const size_t K = c->C == 1 ? 16 : 32, pad = kTcRows;
         if (e == cudaSuccess) e = alloc(&d.qtile, (c->nq_cap + pad - 1) / pad * pad * K * 2);
         if (e == cudaSuccess) e = alloc(&d.ctile, (npix + pad - 1) / pad * pad * K * 2);
+        if (e == cudaSuccess) e = alloc(&d.lists, seed_list_words(c->nq_cap, npix));
         if (e == cudaSuccess) e = alloc(&d.err, 1);
         if (e == cudaSuccess) e = cudaMemset(d.err, 0, sizeof(int));
     }
@@ -1701,16 +1575,13 @@ ff_status ff_seed_knn(ff_ctx *c, ff_dir dir, int32_t *idx_out, int32_t *dist_out
     if (!idx_out || !dist_out) return fail(c, FF_EINVAL, "NULL output");
     DeviceGuard guard(c->device);
     const int d = (int)dir, W = c->fw[0], H = c->fh[0];
-    s = launch_seed_knn(c, d, c->feat[d == 0 ? 0 : 1], c->feat[d == 0 ? 1 : 0], W, H);
-    if (s) return s;
-    int WS, HS;
-    level_dims(W, H, c->S - 1, &WS, &HS);
-    const size_t bytes = (size_t)WS * HS * c->cfg.seed_leaf * sizeof(int);
-    if ((s = check_cuda(c, cudaMemcpyAsync(idx_out, c->dir[d].knn_idx, bytes,
-                                           cudaMemcpyDeviceToDevice, c->stream), "copy knn")))
-        return s;
-    return check_cuda(c, cudaMemcpyAsync(dist_out, c->dir[d].knn_dist, bytes,
-                                         cudaMemcpyDeviceToDevice, c->stream), "copy knn");
+    KnnOut out{};
+    out.leaf = c->cfg.seed_leaf;
+    out.idx = idx_out;
+    out.dist = dist_out;
+    const uint8_t *fs = c->feat[d == 0 ? 0 : 1], *fd = c->feat[d == 0 ? 1 : 0];
+    return c->C == 1 ? launch_seed<1>(c, d, fs, fd, W, H, out)
+                     : launch_seed<3>(c, d, fs, fd, W, H, out);
 }
 
 ff_status ff_seed_knn_static(const int8_t *feat_src0, const int8_t *feat_dst0, int w, int h,
@@ -1887,8 +1758,7 @@ ff_status ff_debug_set(ff_ctx *c, ff_debug_key key, long long value) {
             c->force_timeout = value != 0;
             return FF_OK;
         case FF_DEBUG_SEED_TC:
-            c->seed_tc = value != 0;
-            return FF_OK;
+            return FF_OK;   // the search has one path
         case FF_DEBUG_SWEEP_LANES:
             if (value != 2 && value != 4 && value != 8)
                 return fail(c, FF_EINVAL, "sweep lanes per grid point must be 2, 4 or 8");
@@ -2247,22 +2117,19 @@ ff_status sfail(ff_server *v, ff_status s, const std::string &msg) {
 
 // device bytes ff_create allocates for one context (and so one slot)
 size_t context_bytes(const ff_config &cfg) {
-    const int C = cfg.channels, P = C == 1 ? 16 : 32, K = C == 1 ? 16 : 32;
+    const int C = cfg.channels, P = C == 1 ? 16 : 32;
     const size_t npix = (size_t)cfg.max_width * cfg.max_height;
     int WS, HS;
     level_dims(cfg.max_width, cfg.max_height, cfg.scales - 1, &WS, &HS);
-    const size_t nq = (size_t)WS * HS;
-    (void)C;
+    const size_t nq = (size_t)WS * HS, K = C == 1 ? 16 : 32, pad = kTcRows;
     const int R = rows_per_strip(8);
     const size_t edge = (size_t)((cfg.max_height + R - 1) / R) * cfg.max_width;
     size_t b = 2 * level_offset(cfg.max_width, cfg.max_height, P, cfg.scales);   // features
     b += 2 * npix * C + 3 * npix * 4 + npix;                                    // staging
     b += npix * (4 + 4 + 1);                                                    // region scratch
-    const size_t pad = kTcRows;
-    const size_t dir = npix * 4 * 4 + edge * 8 + FF_MAX_SCALES * kMaxIters * 4 +
-                       nq * FF_MAX_LEAF * 8 + nq * kMaxChunks * 8 * 8 + nq * K * 2 + nq * 4 +
-                       nq * kMaxChunks * 4 + npix * K * 2 + 4 +
-                       ((nq + pad - 1) / pad + (npix + pad - 1) / pad) * pad * K * 2;   // tiles
+    const size_t seed = ((nq + pad - 1) / pad + (npix + pad - 1) / pad) * pad * K * 2 +
+                        seed_list_words(nq, npix) * 4;
+    const size_t dir = npix * 4 * 4 + edge * 8 + FF_MAX_SCALES * kMaxIters * 4 + 4 + seed;
     return b + kNumDirs * dir;
 }
 

@@ -1,18 +1,40 @@
-// ff_seed_tc.cuh - the seeding search's full pass on the 5th-generation
-// tensor cores (tcgen05, accumulators in tensor memory).  Same contraction
-// and output as k_seed_mma (Sec. 3.1 Eq. 1 / Sec. 3.2 Eq. 4 read as an exact
-// top-8 by (|q - c|^2, index)); only the machinery differs.
+// ff_seed_tc.cuh - the seeding search (arXiv 1703.02563, Sec. 3.1 Eq. 1 and
+// Sec. 3.2 Eq. 4: the l candidates of every coarsest-grid point) on the
+// 5th-generation tensor cores (tcgen05, accumulators in tensor memory).
+//
+// The exact top-8 of a query q by (|q - c|^2, index) only needs, per query, the
+// ranking of key(c) = |c|^2 - 2 q.c, since |q|^2 is common.  The keys of all
+// (query, candidate) pairs are one matrix product -- the one dense contraction
+// of the method -- computed exactly on the bf16 tensor cores with FP32
+// accumulation:
+//   query row     = (-2 q_1 .. -2 q_D, 65536, 256, 1, 0 ..)
+//   candidate row = (  c_1 ..   c_D,  h2,  h1, h0, 0 ..),  |c|^2 = h2 65536 + h1 256 + h0
+// Every entry is an integer of magnitude <= 256 or a power of two (exact in
+// bf16), every product is exact, and every partial sum stays below 2^24 in
+// magnitude, so FP32 accumulation in any order returns the key exactly.
+//
+// The product is reduced where it is made: k_seed_tc keeps, per query, the
+// eight tiles of 128 consecutive candidates with the least (least key, tile).
+// They hold the top 8.  For take x = (k, i) of the top 8 in tile t outside
+// them: each of the eight has a candidate of key <= (t's least key) <= k, and
+// where that key equals k its tile, hence its index, comes before x's; so
+// eight candidates come before x, which is not in the top 8.  k_seed_pick
+// then ranks those 1024 candidates exactly.
 #pragma once
 
 #include <cuda_bf16.h>
 
 #include "ff_kernels.cuh"
-#include "ff_seed.cuh"   // key_less, reg_insert
 
 namespace ffk {
 
 constexpr int kTcRows = 128;    // queries per CTA (MMA M) and candidates per tile (MMA N)
-constexpr int kTcStages = 4;    // candidate tiles in flight in shared memory
+constexpr int kTcStages = 4;    // candidate tiles in flight per accumulator
+// A tile's entry in a query's list: least key + kTcKeyBias (21 bits: keys are
+// -|q|^2 .. 3 * 27 * 128^2) above the tile's number in the list (11 bits).
+constexpr int kTcKeyBias = 27 * 128 * 128;
+constexpr int kTcTileBits = 11;
+constexpr int kTcChunkTiles = 1 << kTcTileBits;   // tiles of a chunk, at most
 
 // Byte offset of element (r, k) in a tile of 128 rows x K bf16 laid out for
 // the tensor core without swizzling: 8-row x 16-byte core matrices, the K
@@ -21,29 +43,54 @@ __host__ __device__ constexpr int tc_tile_offset(int r, int k, int K) {
     return (r >> 3) * (K * 16) + (k >> 3) * 128 + (r & 7) * 16 + (k & 7) * 2;
 }
 
-// Row-major bf16 rows of K (n of them) -> 128-row tiles in the layout above.
-// Rows n .. to the next multiple of 128 are padding: zeros, or for
-// candidates a +inf at position dh2, so that their keys are +inf.
-template <int K>
-__global__ void k_seed_tile(const __nv_bfloat16 *__restrict__ rows, int n, int dh2,
-                            uint8_t *__restrict__ tiles) {
-    const int npad = (n + kTcRows - 1) / kTcRows * kTcRows;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;   // one 16-byte piece
-    if (j >= npad * (K / 8)) return;
-    const int r = j / (K / 8), kg = j - r * (K / 8);
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if (r < n) {
-        v = reinterpret_cast<const uint4 *>(rows + (size_t)r * K)[kg];
-    } else if (dh2 >= 0 && dh2 / 8 == kg) {
-        __align__(16) __nv_bfloat16 z[8];
+// The rows above (K = 16 gray, 32 Lab) in tiles of 128, straight from the
+// level-0 features: the ncand candidates of the stride grid (padded with rows
+// whose h2 is +inf, so that their keys are), then the nq queries (padded with
+// zero rows).
+template <int C>
+__global__ void __launch_bounds__(128)
+    k_seed_prep(const uint8_t *__restrict__ fq, const uint8_t *__restrict__ fc, int W, int N,
+                int WS, int nq, int stride, int Wc, int ncand, uint8_t *__restrict__ qtile,
+                uint8_t *__restrict__ ctile) {
+    constexpr int D = 9 * C, K = C == 1 ? 16 : 32, P = Geo<C>::P;
+    const int nct = (ncand + kTcRows - 1) / kTcRows;
+    const bool query = (int)blockIdx.x >= nct;
+    const int t = query ? blockIdx.x - nct : blockIdx.x, r = t * kTcRows + threadIdx.x;
+    uint32_t w[P / 4];
 #pragma unroll
-        for (int e = 0; e < 8; e++)
-            z[e] = (kg * 8 + e == dh2) ? __float2bfloat16(__int_as_float(0x7f800000))
-                                       : __int2bfloat16_rn(0);
-        v = *reinterpret_cast<const uint4 *>(z);
+    for (int k = 0; k < P / 4; k++) w[k] = 0;
+    const bool real = r < (query ? nq : ncand);
+    if (real) {
+        const int wd = query ? WS : Wc, y = r / wd, x = r - y * wd, step = query ? N : stride;
+        const uint4 *src = reinterpret_cast<const uint4 *>(
+            (query ? fq : fc) + ((size_t)y * step * W + (size_t)x * step) * P);
+#pragma unroll
+        for (int v = 0; v < P / 16; v++) {
+            const uint4 u = __ldg(src + v);
+            w[4 * v] = u.x, w[4 * v + 1] = u.y, w[4 * v + 2] = u.z, w[4 * v + 3] = u.w;
+        }
     }
-    uint8_t *tile = tiles + (size_t)(r / kTcRows) * kTcRows * K * 2;
-    *reinterpret_cast<uint4 *>(tile + tc_tile_offset(r % kTcRows, kg * 8, K)) = v;
+    int nn = 0;
+#pragma unroll
+    for (int k = 0; k < P / 4; k++) nn = __dp4a((int)w[k], (int)w[k], nn);
+    __align__(16) __nv_bfloat16 row[K];
+#pragma unroll
+    for (int d = 0; d < D; d++) {
+        const int v = (int)(int8_t)(w[d >> 2] >> (8 * (d & 3)));
+        row[d] = __int2bfloat16_rn(query ? -2 * v : v);
+    }
+    row[D] = real ? __int2bfloat16_rn(query ? 65536 : nn >> 16)
+                  : (query ? __int2bfloat16_rn(0)
+                           : __float2bfloat16(__int_as_float(0x7f800000)));
+    row[D + 1] = __int2bfloat16_rn(!real ? 0 : (query ? 256 : (nn >> 8) & 255));
+    row[D + 2] = __int2bfloat16_rn(!real ? 0 : (query ? 1 : nn & 255));
+#pragma unroll
+    for (int d = D + 3; d < K; d++) row[d] = __int2bfloat16_rn(0);
+    uint8_t *tile = (query ? qtile : ctile) + (size_t)t * kTcRows * K * 2;
+#pragma unroll
+    for (int kg = 0; kg < K / 8; kg++)
+        *reinterpret_cast<uint4 *>(tile + tc_tile_offset(threadIdx.x, kg * 8, K)) =
+            reinterpret_cast<const uint4 *>(row)[kg];
 }
 
 __device__ __forceinline__ uint32_t tc_smem(const void *p) {
@@ -61,10 +108,10 @@ __device__ __forceinline__ void mbar_init(uint64_t *m, int count) {
 __device__ __forceinline__ bool mbar_test(uint64_t *m, uint32_t parity) {
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\n\t"
+        "{\n\t.reg .pred q;\n\tmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, %3;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(ok)
-        : "r"(tc_smem(m)), "r"(parity)
+        : "r"(tc_smem(m)), "r"(parity), "r"(100000)
         : "memory");
     return ok != 0;
 }
@@ -103,67 +150,86 @@ __device__ __forceinline__ void bulk_copy(void *dst, const void *src, uint32_t b
 
 template <int KS>
 __host__ __device__ constexpr int tc_seed_smem_bytes() {
-    return kTcRows * 16 * KS * 2 * (1 + kTcStages) + 8 * 32 * 32 * 4;
+    return kTcRows * 16 * KS * 2 * (1 + 2 * kTcStages);
 }
 
-// 64 consecutive 32-bit columns of this warp's 32 tensor-memory lanes
-__device__ __forceinline__ void tmem_ld64(uint32_t *r, uint32_t taddr) {
+// The least of 128 consecutive 32-bit columns of each of this warp's 32
+// tensor-memory lanes, reduced by the load itself; the loaded columns are not
+// used.
+__device__ __forceinline__ float tmem_min128(uint32_t taddr) {
+    [[maybe_unused]] uint32_t r[128];
+    uint32_t least;
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63}, [%64];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        "tcgen05.ld.red.sync.aligned.32x32b.x128.min.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8,"
+        " %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25,"
+        " %26, %27, %28, %29, %30, %31, %32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42"
+        ", %43, %44, %45, %46, %47, %48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %5"
+        "9, %60, %61, %62, %63, %64, %65, %66, %67, %68, %69, %70, %71, %72, %73, %74, %75, %"
+        "76, %77, %78, %79, %80, %81, %82, %83, %84, %85, %86, %87, %88, %89, %90, %91, %92, "
+        "%93, %94, %95, %96, %97, %98, %99, %100, %101, %102, %103, %104, %105, %106, %107, %"
+        "108, %109, %110, %111, %112, %113, %114, %115, %116, %117, %118, %119, %120, %121, %"
+        "122, %123, %124, %125, %126, %127}, %128, [%129];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+          "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+          "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
+          "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
+          "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63]),
+          "=r"(r[64]), "=r"(r[65]), "=r"(r[66]), "=r"(r[67]), "=r"(r[68]), "=r"(r[69]), "=r"(r[70]), "=r"(r[71]),
+          "=r"(r[72]), "=r"(r[73]), "=r"(r[74]), "=r"(r[75]), "=r"(r[76]), "=r"(r[77]), "=r"(r[78]), "=r"(r[79]),
+          "=r"(r[80]), "=r"(r[81]), "=r"(r[82]), "=r"(r[83]), "=r"(r[84]), "=r"(r[85]), "=r"(r[86]), "=r"(r[87]),
+          "=r"(r[88]), "=r"(r[89]), "=r"(r[90]), "=r"(r[91]), "=r"(r[92]), "=r"(r[93]), "=r"(r[94]), "=r"(r[95]),
+          "=r"(r[96]), "=r"(r[97]), "=r"(r[98]), "=r"(r[99]), "=r"(r[100]), "=r"(r[101]), "=r"(r[102]), "=r"(r[103]),
+          "=r"(r[104]), "=r"(r[105]), "=r"(r[106]), "=r"(r[107]), "=r"(r[108]), "=r"(r[109]), "=r"(r[110]), "=r"(r[111]),
+          "=r"(r[112]), "=r"(r[113]), "=r"(r[114]), "=r"(r[115]), "=r"(r[116]), "=r"(r[117]), "=r"(r[118]), "=r"(r[119]),
+          "=r"(r[120]), "=r"(r[121]), "=r"(r[122]), "=r"(r[123]), "=r"(r[124]), "=r"(r[125]), "=r"(r[126]), "=r"(r[127]),
+          "=r"(least)
         : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    asm volatile("" : "+r"(least));
+    return __uint_as_float(least);
 }
 
 // Per CTA: 128 queries (tensor-memory lanes; epilogue thread = query row)
-// against one chunk of candidates, 128 per tile.  Warp 8 allocates tensor
-// memory and streams candidate tiles into a 4-stage ring with bulk copies;
-// warp 9 issues the K/16 MMAs of each tile into one of two 128-column
-// accumulators; warps 0-7 read their rows' keys per tile with tcgen05.ld
-// (warps w and w + 4: the same rows, the first and the second 64 columns)
-// and keep each query's top-8 by (key, index) in registers, key
-// entering only at or below min(the query's bound t0, its 8th key) (a key
-// equal to it only while the list's 8th key is larger; keys are exact
-// integers).  All waits are bounded.  Output as k_seed_mma, with two lists
-// per chunk (chunk slots 2 blockIdx.y and 2 blockIdx.y + 1).
+// against one chunk of candidates, 128 per tile; even tiles go through one
+// 128-column accumulator, odd ones through the other, and each has its own
+// issuing warp (4, 5), whose thread keeps four tiles of bulk copies in flight
+// and issues the K/16 MMAs of a tile once its accumulator has been drained.
+// Each thread of the epilogue warps (0-3) takes its row's least key out of the
+// accumulator with one reducing tensor-memory load and puts (least key, tile)
+// into its list of eight.  All waits are bounded.  The list of chunk c and
+// query row q is lists[(c * 128 nqt + q) * 8 ..], empty entries 0xffffffff.
 template <int KS>
-__global__ void __launch_bounds__(320)
-    k_seed_tc(const uint8_t *__restrict__ qtile, const int *__restrict__ qn,
-              const uint8_t *__restrict__ ctile, int NQ, int NC, int chunk, int W, int stride,
-              int Wc, const float *__restrict__ t0, int t0_chunks, int2 *__restrict__ part,
-              int *err, unsigned long long wait_ns) {
+__global__ void __launch_bounds__(192, 2)
+    k_seed_tc(const uint8_t *__restrict__ qtile, const uint8_t *__restrict__ ctile, int nct,
+              int chunk, uint32_t *__restrict__ lists, int *err, unsigned long long wait_ns) {
     constexpr int K = 16 * KS;
     constexpr uint32_t TILE_BYTES = kTcRows * K * 2;
-    constexpr float kEmpty = 3.0e38f;
-    // dynamic shared memory (tc_seed_smem_bytes<KS>()): the query tile, the
-    // candidate ring and each epilogue warp's 32 x 32 key scratch
+    // dynamic shared memory (tc_seed_smem_bytes<KS>()): the query tile and the candidate ring
     extern __shared__ __align__(1024) uint8_t tc_dyn[];
     uint8_t *sA = tc_dyn;
     uint8_t(*sB)[TILE_BYTES] = reinterpret_cast<uint8_t(*)[TILE_BYTES]>(tc_dyn + TILE_BYTES);
-    float(*scr)[32][32] =
-        reinterpret_cast<float(*)[32][32]>(tc_dyn + TILE_BYTES * (1 + kTcStages));   // [8][32][32]
-    __shared__ __align__(8) uint64_t bar_a, full[kTcStages], empty[kTcStages], accf[2], acce[2];
+    __shared__ __align__(8) uint64_t bar_a, full[2 * kTcStages], accf[2], acce[2];
     __shared__ uint32_t taddr_slot;
     __shared__ int abort_flag;
     volatile int *v_abort = &abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int qt = blockIdx.x;
-    const int c0 = blockIdx.y * chunk, c1 = min(c0 + chunk, NC);
-    const int ntiles = (c1 - c0 + kTcRows - 1) / kTcRows;   // chunk is a multiple of 128
+    const int tile0 = blockIdx.y * chunk, ntiles = min(chunk, nct - tile0);
     if (tid == 0) {
         abort_flag = 0;
         mbar_init(&bar_a, 1);
-        for (int s = 0; s < kTcStages; s++) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
+        for (int s = 0; s < 2 * kTcStages; s++) mbar_init(&full[s], 1);
         for (int b = 0; b < 2; b++) {
             mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], 8);
+            mbar_init(&acce[b], 4);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 8) {
+    if (warp == 4) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(
             tc_smem(&taddr_slot)));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -173,38 +239,38 @@ __global__ void __launch_bounds__(320)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t taddr = taddr_slot;
 
-    if (warp == 8) {
-        // ---------------- producer: queries once, then candidate tiles
+    if (warp >= 4) {
+        // ---------------- copies and MMAs of the tiles 2 n + g
+        const int g = warp - 4, mine = (ntiles - g + 1) / 2;
         if (lane == 0) {
-            mbar_expect_tx(&bar_a, TILE_BYTES);
-            bulk_copy(sA, qtile + (size_t)qt * TILE_BYTES, TILE_BYTES, &bar_a);
-            const int tile0 = c0 / kTcRows;
-            for (int t = 0; t < ntiles; t++) {
-                const int s = t % kTcStages;
-                if (t >= kTcStages &&
-                    !mbar_wait(&empty[s], ((t / kTcStages) - 1) & 1, wait_ns, v_abort, err))
-                    break;
-                mbar_expect_tx(&full[s], TILE_BYTES);
-                bulk_copy(sB[s], ctile + (size_t)(tile0 + t) * TILE_BYTES, TILE_BYTES, &full[s]);
+            uint64_t *fullg = full + g * kTcStages;
+            uint8_t(*ring)[TILE_BYTES] = sB + g * kTcStages;
+            const uint8_t *src = ctile + (size_t)(tile0 + g) * TILE_BYTES;
+            auto copy = [&](int n) {
+                mbar_expect_tx(&fullg[n % kTcStages], TILE_BYTES);
+                bulk_copy(ring[n % kTcStages], src + (size_t)n * 2 * TILE_BYTES, TILE_BYTES,
+                          &fullg[n % kTcStages]);
+            };
+            if (g == 0) {
+                mbar_expect_tx(&bar_a, TILE_BYTES);
+                bulk_copy(sA, qtile + (size_t)qt * TILE_BYTES, TILE_BYTES, &bar_a);
             }
-        }
-    } else if (warp == 9) {
-        // ---------------- MMA issuer
-        if (lane == 0 && mbar_wait(&bar_a, 0, wait_ns, v_abort, err)) {
+            for (int n = 0; n < min(kTcStages, mine); n++) copy(n);
             // kind::f16, bf16 x bf16 -> f32, both K-major, N = 128, M = 128
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                        ((uint32_t)(kTcRows >> 3) << 17) |
                                        ((uint32_t)(kTcRows >> 4) << 24);
-            for (int t = 0; t < ntiles; t++) {
-                const int s = t % kTcStages, b = t & 1;
-                if (!mbar_wait(&full[s], (t / kTcStages) & 1, wait_ns, v_abort, err)) break;
-                if (t >= 2 && !mbar_wait(&acce[b], ((t >> 1) - 1) & 1, wait_ns, v_abort, err)) break;
+            const uint32_t d = taddr + (uint32_t)(g * kTcRows);
+            const bool have_a = mbar_wait(&bar_a, 0, wait_ns, v_abort, err);
+            for (int n = 0; n < mine && have_a; n++) {
+                const int s = n % kTcStages;
+                if (!mbar_wait(&fullg[s], (n / kTcStages) & 1, wait_ns, v_abort, err)) break;
+                if (n >= 1 && !mbar_wait(&acce[g], (n - 1) & 1, wait_ns, v_abort, err)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d = taddr + (uint32_t)(b * kTcRows);
 #pragma unroll
                 for (int ks = 0; ks < KS; ks++) {
                     const uint64_t da = tc_desc(tc_smem(sA) + ks * 256, 128, K * 16);
-                    const uint64_t db = tc_desc(tc_smem(sB[s]) + ks * 256, 128, K * 16);
+                    const uint64_t db = tc_desc(tc_smem(ring[s]) + ks * 256, 128, K * 16);
                     asm volatile(
                         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
@@ -212,98 +278,198 @@ __global__ void __launch_bounds__(320)
                 }
                 asm volatile(
                     "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
-                        "r"(tc_smem(&empty[s]))
+                        "r"(tc_smem(&accf[g]))
                     : "memory");
-                asm volatile(
-                    "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::
-                        "r"(tc_smem(&accf[b]))
-                    : "memory");
+                // tile n - 1 has been drained, so its product is done with its stage
+                if (n >= 1 && n - 1 + kTcStages < mine) copy(n - 1 + kTcStages);
             }
         }
     } else {
-        // ---------------- epilogue: warps w and w + 4 share tensor-memory lanes
-        // 32 (w mod 4) .. +31 (thread = query row) and take the first and the
-        // second 64 keys of each tile: two lists per query, merged later
-        const int quarter = warp & 3, half = warp >> 2;
-        const int row = quarter * 32 + lane, q = qt * kTcRows + row;
-        float tinit = kEmpty;
-        if (t0 && q < NQ)
-            for (int c = 0; c < t0_chunks; c++) tinit = fminf(tinit, __ldg(t0 + (size_t)c * NQ + q));
-        float lk[8];
-        int li[8];
+        // ---------------- epilogue: warp w reads tensor-memory lanes 32 w .. +31
+        // (thread = query row)
+        const uint32_t ta = taddr + ((uint32_t)(warp * 32) << 16);
+        uint32_t l[8];
 #pragma unroll
-        for (int e = 0; e < 8; e++) {
-            lk[e] = kEmpty;
-            li[e] = 0x7fffffff;
-        }
+        for (int e = 0; e < 8; e++) l[e] = 0xffffffffu;
         for (int t = 0; t < ntiles; t++) {
-            const int b = t & 1;
-            if (!mbar_wait(&accf[b], (t >> 1) & 1, wait_ns, v_abort, err)) break;
+            const int g = t & 1;
+            if (!mbar_wait(&accf[g], (t >> 1) & 1, wait_ns, v_abort, err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int base = c0 + t * kTcRows;
-            // this warp's 64 keys of the tile for its row
-            uint32_t r[64];
-            const uint32_t ta = taddr + ((uint32_t)(quarter * 32) << 16) +
-                                (uint32_t)(b * kTcRows + half * 64);
-            tmem_ld64(r, ta);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            // bound of this row: a key equal to it counts only while the list's
-            // 8th key is larger
-            float tq = fminf(lk[7], tinit);
-            float thr = lk[7] > tq ? tq + 1.0f : tq;
-#pragma unroll
-            for (int cc = 0; cc < 64; cc += 32) {
-                float mn = __uint_as_float(r[cc]);
-#pragma unroll
-                for (int j = 1; j < 32; j++) mn = fminf(mn, __uint_as_float(r[cc + j]));
-                if (mn < thr) {
-                    // rare: the hits of these 32 keys, in column order, through
-                    // this lane's scratch column
-                    uint32_t mask = 0;
-#pragma unroll
-                    for (int j = 0; j < 32; j++) {
-                        const float key = __uint_as_float(r[cc + j]);
-                        scr[warp][j][lane] = key;
-                        mask |= (key < thr ? 1u : 0u) << j;
-                    }
-                    while (mask) {
-                        const int j = __ffs(mask) - 1;
-                        mask &= mask - 1;
-                        const float key = scr[warp][j][lane];
-                        if (key < thr) {
-                            const int ord = base + half * 64 + cc + j;
-                            if (key_less(key, ord, lk[7], li[7])) reg_insert(lk, li, key, ord);
-                            tq = fminf(lk[7], tinit);
-                            thr = lk[7] > tq ? tq + 1.0f : tq;
-                        }
-                    }
-                }
-            }
+            const float least = tmem_min128(ta + (uint32_t)(g * kTcRows));
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acce[b]);
-        }
-        if (q < NQ && !*v_abort) {
-            const int qq = qn[q];
-            int2 *dst = part + ((size_t)(2 * blockIdx.y + half) * NQ + q) * 8;
+            if (lane == 0) mbar_arrive(&acce[g]);
+            // key + bias in the low mantissa bits of 2^23 + key + bias (exact)
+            uint32_t x = (__float_as_uint(least + (float)(8388608 + kTcKeyBias)) << kTcTileBits) +
+                         (uint32_t)t;
 #pragma unroll
             for (int e = 0; e < 8; e++) {
-                if (li[e] == 0x7fffffff) {
-                    dst[e] = make_int2(0x7fffffff, 0x7fffffff);
-                } else {
-                    const int ci = li[e];
-                    const int idx = (ci / Wc) * stride * W + (ci % Wc) * stride;
-                    dst[e] = make_int2((int)lk[e] + qq, idx);
-                }
+                const uint32_t lo = min(l[e], x);
+                x = max(l[e], x);
+                l[e] = lo;
             }
         }
+        const size_t row = ((size_t)blockIdx.y * gridDim.x + qt) * kTcRows + warp * 32 + lane;
+        uint4 *dst = reinterpret_cast<uint4 *>(lists + row * 8);
+        dst[0] = make_uint4(l[0], l[1], l[2], l[3]);
+        dst[1] = make_uint4(l[4], l[5], l[6], l[7]);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 8) {
+    if (warp == 4) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(taddr));
     }
+}
+
+__device__ __forceinline__ bool lex_less(int d, int i, int D, int I) {
+    return d < D || (d == D && i < I);
+}
+
+// A query's list across a warp: lane e holds its e-th best (distance, index).
+struct KnnList {
+    int D, I;
+};
+__device__ __forceinline__ void knn_insert(KnnList &l, int d, int i, int lane) {
+    const bool less = lex_less(d, i, l.D, l.I);
+    const int uD = __shfl_up_sync(0xffffffffu, l.D, 1), uI = __shfl_up_sync(0xffffffffu, l.I, 1);
+    if (less) {
+        const bool here = lane == 0 || !lex_less(d, i, uD, uI);
+        l.D = here ? d : uD;
+        l.I = here ? i : uI;
+    }
+}
+// Puts every lane's (d, i) into the list that belongs among its first eight
+// and does not come behind (capD, capI).  The eighth entry is looked at after
+// each insertion, so that of many equal distances (flat image regions) only
+// the first few are inserted.
+__device__ __forceinline__ void knn_take(KnnList &l, int d, int i, int lane, int capD, int capI) {
+    unsigned m = 0xffffffffu;
+    for (;;) {
+        int D = __shfl_sync(0xffffffffu, l.D, 7), I = __shfl_sync(0xffffffffu, l.I, 7);
+        if (lex_less(capD, capI, D, I)) D = capD, I = capI;
+        m &= __ballot_sync(0xffffffffu, lex_less(d, i, D, I));
+        if (!m) return;
+        const int s = __ffs(m) - 1;
+        m &= m - 1;
+        knn_insert(l, __shfl_sync(0xffffffffu, d, s), __shfl_sync(0xffffffffu, i, s), lane);
+    }
+}
+
+// What becomes of a finished list: its first `leaf` entries to the caller
+// (idx, dist), and, for a match, the one of lowest matching error at the
+// coarsest scale (Eq. 1), the earlier rank on ties, as the point's flow.
+struct KnnOut {
+    int leaf;
+    int *idx, *dist;               // [queries][leaf], or NULL
+    const uint8_t *f1L, *f2L;      // coarsest level
+    int W, H, L, WL, HL;
+    uint32_t *flow;                // [queries], or NULL
+    int *cost;
+};
+template <int C>
+__device__ __forceinline__ void knn_finish(const KnnOut &o, int q, int lane, KnnList l) {
+    constexpr int P = Geo<C>::P;
+    const bool ok = lane < o.leaf && l.D != 0x7fffffff;
+    if (o.idx && lane < o.leaf) {
+        o.idx[(size_t)q * o.leaf + lane] = ok ? l.I : -1;
+        o.dist[(size_t)q * o.leaf + lane] = ok ? l.D : -1;
+    }
+    if (!o.flow) return;
+    const int gy = q / o.WL, gx = q - gy * o.WL;
+    const int px = gx << o.L, py = gy << o.L;
+    uint32_t f = kFlowInvalid;
+    int e = kCostInvalid;
+    if (ok) {
+        uint32_t qw[P / 4];
+#pragma unroll
+        for (int w = 0; w < P / 4; w++) qw[w] = ldg32(o.f1L + (size_t)q * P + 4 * w);
+        int fx = 8 * (l.I % o.W - px), fy = 8 * (l.I / o.W - py);
+        clamp_flow(o.W, o.H, px, py, fx, fy);
+        e = sad_full<C>(o.f2L, make_tap<P>(px, py, fx, fy, o.L, o.WL, o.HL), qw);
+        f = pack_flow(fx, fy);
+    }
+    const int best = __reduce_min_sync(0xffffffffu, e);
+    const int win = __ffs(__ballot_sync(0xffffffffu, e == best)) - 1;
+    if (lane == win) {
+        o.flow[q] = f;
+        o.cost[q] = e;
+    }
+}
+
+// A query's tile lists -> its top 8 (and, for a match, its coarsest flow); one
+// warp per query.  The eight tiles of least (key, tile) come from its nch
+// lists; the eighth's least key bounds the eighth distance, so few of their
+// 1024 candidates are ever inserted.
+template <int C>
+__global__ void __launch_bounds__(128)
+    k_seed_pick(const uint8_t *__restrict__ fq, const uint8_t *__restrict__ fc, int W, int N,
+                int WS, int nq, int stride, int Wc, int ncand, const uint32_t *__restrict__ lists,
+                int nqt, int nch, int chunk, const KnnOut out) {
+    constexpr int P = Geo<C>::P, NV = P / 16, NW = Geo<C>::NW;
+    constexpr unsigned FULL = 0xffffffffu;
+    const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (q >= nq) return;
+    uint32_t qw[4 * NV];
+    {
+        const int gy = q / WS, gx = q - gy * WS;
+        const uint4 *src = reinterpret_cast<const uint4 *>(
+            fq + ((size_t)gy * N * W + (size_t)gx * N) * P);
+#pragma unroll
+        for (int v = 0; v < NV; v++) {
+            const uint4 u = __ldg(src + v);
+            qw[4 * v] = u.x, qw[4 * v + 1] = u.y, qw[4 * v + 2] = u.z, qw[4 * v + 3] = u.w;
+        }
+    }
+    int qn = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) qn = __dp4a((int)qw[w], (int)qw[w], qn);
+    // the eight tiles (D: least key + bias, I: tile), four lists at a time
+    KnnList best{0x7fffffff, 0x7fffffff};
+    for (int c0 = 0; c0 < nch; c0 += 4) {
+        const int c = c0 + (lane >> 3);
+        int d = 0x7fffffff, t = 0x7fffffff;
+        if (c < nch) {
+            const uint32_t x = __ldg(lists + ((size_t)c * nqt * kTcRows + q) * 8 + (lane & 7));
+            if (x != 0xffffffffu) {
+                d = (int)(x >> kTcTileBits);
+                t = c * chunk + (int)(x & ((1u << kTcTileBits) - 1));
+            }
+        }
+        knn_take(best, d, t, lane, 0x7fffffff, 0x7fffffff);
+    }
+    const int D7 = __shfl_sync(FULL, best.D, 7);
+    const int bD = D7 == 0x7fffffff ? D7 : D7 - kTcKeyBias + qn;
+    KnnList l{0x7fffffff, 0x7fffffff};
+    for (int k = 0; k < 8; k++) {
+        const int t = __shfl_sync(FULL, best.I, k);
+        if (t == 0x7fffffff) break;
+        uint4 r[4][NV];
+        int idx[4];
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int o = min(t * kTcRows + 32 * j + lane, ncand - 1);
+            const int cy = o / Wc, cx = o - cy * Wc;
+            idx[j] = cy * stride * W + cx * stride;
+#pragma unroll
+            for (int v = 0; v < NV; v++)
+                r[j][v] = __ldg(reinterpret_cast<const uint4 *>(fc + (size_t)idx[j] * P) + v);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            int dot = 0, nn = 0;
+#pragma unroll
+            for (int w = 0; w < NW; w++) {
+                const uint32_t cw = reinterpret_cast<const uint32_t *>(&r[j][0])[w];
+                dot = __dp4a((int)cw, (int)qw[w], dot);
+                nn = __dp4a((int)cw, (int)cw, nn);
+            }
+            const int d = nn + qn - 2 * dot;
+            const bool real = t * kTcRows + 32 * j + lane < ncand;
+            knn_take(l, real ? d : 0x7fffffff, idx[j], lane, bD, 0x7fffffff);
+        }
+    }
+    knn_finish<C>(out, q, lane, l);
 }
 
 }  // namespace ffk

@@ -1,0 +1,66 @@
+"""The seeding search (csrc/ff_seed_tc.cuh: tiles on the tensor cores, then the
+eight best tiles' candidates) against the oracle: all integers, tolerance 0."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_1703_02563_gb300 import ff
+
+pytestmark = pytest.mark.gpu
+
+
+def _frames(kind, C, W, H, seed):
+    r = np.random.default_rng(seed)
+    if kind == "noise":        # no structure
+        return r.integers(0, 256, (2, C, H, W), dtype=np.uint8)
+    if kind == "constant":     # every distance is 0: only the index ranks
+        return np.full((2, C, H, W), 77, np.uint8)
+    if kind == "stripes":      # few different vectors, many candidates each
+        f = np.zeros((2, C, H, W), np.uint8)
+        f[..., (np.arange(W) // 16) % 2 == 1] = 200
+        f[1] = np.roll(f[1], 5, axis=-1)
+        return f
+    smooth = r.integers(0, 256, (2, C, H // 8 + 2, W // 8 + 2)).astype(np.float64)
+    f = np.kron(smooth, np.ones((1, 1, 8, 8)))[:, :, :H, :W]
+    f = f + r.integers(-6, 7, f.shape)
+    return np.clip(f, 0, 255).astype(np.uint8)
+
+
+CASES = [("smooth", 1, 1, 1, 1, 8, 1), ("smooth", 3, 31, 1, 1, 8, 1), ("smooth", 1, 33, 1, 2, 4, 1),
+         ("smooth", 3, 32, 32, 2, 8, 1), ("smooth", 1, 41, 25, 2, 8, 1),
+         # several chunks of tiles, ragged last tile; an odd stride
+         ("smooth", 3, 430, 310, 4, 8, 1), ("smooth", 1, 257, 190, 3, 5, 3),
+         # noise, where no two candidates are near:
+         # one and several tiles of 128 queries, one chunk and many
+         ("noise", 3, 256, 192, 3, 8, 1), ("noise", 1, 256, 192, 4, 8, 1),
+         ("noise", 1, 300, 200, 2, 8, 1), ("noise", 3, 400, 300, 3, 8, 2),
+         ("constant", 1, 200, 150, 3, 8, 1), ("stripes", 3, 160, 120, 3, 8, 1),
+         ("stripes", 1, 200, 90, 2, 3, 1)]
+
+
+@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", CASES)
+@pytest.mark.parametrize("tc", [1, 0])
+def test_seed_lists_equal_the_oracle(kind, C, W, H, S, leaf, stride, tc):
+    import torch
+    f = _frames(kind, C, W, H, W * 1000 + H)
+    ctx = ff.Context(ff.Config(channels=C, scales=S, iters=1, seed_leaf=leaf, seed_stride=stride,
+                               max_width=W + 3, max_height=H + 1))
+    ff.ff_debug_set(ctx.ctx, ff.FF_DEBUG_SEED_TC, tc)
+    for slot in (0, 1):
+        ctx.features(slot, torch.from_numpy(f[slot]).cuda())
+    f1, f2 = (O.features_all(f[k], S)[0] for k in (0, 1))
+    for d, (a, b) in enumerate(((f1, f2), (f2, f1))):
+        idx, dist = ctx.seed_knn(d)
+        ridx, rdist = O.seed_knn(a, b, S, leaf, stride)
+        np.testing.assert_array_equal(idx.cpu().numpy(), ridx)
+        np.testing.assert_array_equal(dist.cpu().numpy(), rdist)
+    # and a match seeded by it: the rerank at the coarsest scale
+    flow, cost = ctx.match(0, 1, until_level=S - 1, until_sweeps=0)
+    P = O.Params(channels=C, scales=S, iters=1, seed_leaf=leaf, seed_stride=stride)
+    rf, rc, _ = O.match(P, f[0], f[1], 0, 1, until_level=S - 1, until_sweeps=0)
+    np.testing.assert_array_equal(flow.cpu().numpy(), rf)
+    np.testing.assert_array_equal(cost.cpu().numpy(), rc)
+    ctx.sync()
+    ctx.close()
