@@ -778,9 +778,12 @@ void seed_geometry(int nq, int ncand, int sms, int *nchunks, int *chunk) {
 // How the seeding's product is split: nqt tiles of 128 queries by nch chunks of
 // `chunk` tiles of 128 candidates.  Two CTAs share an SM, so `slots` run at
 // once; among the chunk counts the one whose waves take the fewest tiles is
-// taken, a CTA's start counting as kTcStartTiles.  (One wave of 5 chunks at
-// 1024x436 leaves 29 of 304 slots idle, two waves of 11 leave 3.)
-constexpr int kTcStartTiles = 24, kTcMaxChunks = 16, kTcMaxSlots = 512;
+// taken, where a CTA's start counts as kTcStartTiles and every four lists that
+// k_seed_pick has to merge as kTcMergeTiles.  (One wave of 5 chunks at 1024x436
+// leaves 29 of 304 slots idle, two waves of 11 leave 3.  At 128x96 50 chunks
+// kept every SM busy, but their merge took 25 us against 16.5 now; the search
+// there 34 against 29 us.)
+constexpr int kTcStartTiles = 24, kTcMergeTiles = 15, kTcMaxChunks = 16, kTcMaxSlots = 512;
 struct SeedSplit {
     int nqt, nct, nch, chunk;
 };
@@ -795,7 +798,8 @@ SeedSplit seed_split(size_t nq, size_t ncand, int slots) {
     z.nch = 0;
     for (int n = least; n <= most; n++) {
         const long long waves = ((long long)z.nqt * n + slots - 1) / slots;
-        const long long t = waves * ((z.nct + n - 1) / n + kTcStartTiles);
+        const long long t = waves * ((z.nct + n - 1) / n + kTcStartTiles) +
+                            (n + 3) / 4 * kTcMergeTiles;
         if (z.nch == 0 || t < best) best = t, z.nch = n;
     }
     z.chunk = (z.nct + z.nch - 1) / z.nch;

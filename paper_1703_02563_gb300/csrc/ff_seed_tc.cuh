@@ -356,6 +356,23 @@ __device__ __forceinline__ void knn_take(KnnList &l, int d, int i, int lane, int
     }
 }
 
+// The warp's (d, i) pairs in order, through the warp's 32 words of buf (the
+// empty ones, d = 0x7fffffff, last).
+__device__ __forceinline__ KnnList knn_sort(int d, int i, int2 *buf, int lane) {
+    int r = 0;
+#pragma unroll
+    for (int k = 0; k < 32; k++) {
+        const int D = __shfl_sync(0xffffffffu, d, k), I = __shfl_sync(0xffffffffu, i, k);
+        r += lex_less(D, I, d, i) || (D == d && I == i && k < lane);
+    }
+    __syncwarp();
+    buf[r] = make_int2(d, i);
+    __syncwarp();
+    const int2 e = buf[lane];
+    __syncwarp();
+    return KnnList{e.x, e.y};
+}
+
 // What becomes of a finished list: its first `leaf` entries to the caller
 // (idx, dist), and, for a match, the one of lowest matching error at the
 // coarsest scale (Eq. 1), the earlier rank on ties, as the point's flow.
@@ -400,7 +417,7 @@ __device__ __forceinline__ void knn_finish(const KnnOut &o, int q, int lane, Knn
 // A query's tile lists -> its top 8 (and, for a match, its coarsest flow); one
 // warp per query.  The eight tiles of least (key, tile) come from its nch
 // lists; the eighth's least key bounds the eighth distance, so few of their
-// 1024 candidates are ever inserted.
+// 1024 candidates are kept: those are collected and sorted once.
 template <int C>
 __global__ void __launch_bounds__(128)
     k_seed_pick(const uint8_t *__restrict__ fq, const uint8_t *__restrict__ fc, int W, int N,
@@ -408,7 +425,9 @@ __global__ void __launch_bounds__(128)
                 int nqt, int nch, int chunk, const KnnOut out) {
     constexpr int P = Geo<C>::P, NV = P / 16, NW = Geo<C>::NW;
     constexpr unsigned FULL = 0xffffffffu;
+    __shared__ int2 s_buf[4][32];
     const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    int2 *buf = s_buf[threadIdx.x >> 5];
     if (q >= nq) return;
     uint32_t qw[4 * NV];
     {
@@ -424,7 +443,7 @@ __global__ void __launch_bounds__(128)
     int qn = 0;
 #pragma unroll
     for (int w = 0; w < NW; w++) qn = __dp4a((int)qw[w], (int)qw[w], qn);
-    // the eight tiles (D: least key + bias, I: tile), four lists at a time
+    // the eight tiles (D: least key + bias, I: tile); a list is sorted
     KnnList best{0x7fffffff, 0x7fffffff};
     for (int c0 = 0; c0 < nch; c0 += 4) {
         const int c = c0 + (lane >> 3);
@@ -436,11 +455,16 @@ __global__ void __launch_bounds__(128)
                 t = c * chunk + (int)(x & ((1u << kTcTileBits) - 1));
             }
         }
-        knn_take(best, d, t, lane, 0x7fffffff, 0x7fffffff);
+        if (c0 == 0)
+            best = nch == 1 ? KnnList{d, t} : knn_sort(d, t, buf, lane);
+        else
+            knn_take(best, d, t, lane, 0x7fffffff, 0x7fffffff);
     }
     const int D7 = __shfl_sync(FULL, best.D, 7);
-    const int bD = D7 == 0x7fffffff ? D7 : D7 - kTcKeyBias + qn;
+    // (bD, bI): nothing behind it belongs to the top 8
+    int bD = D7 == 0x7fffffff ? D7 : D7 - kTcKeyBias + qn, bI = 0x7fffffff;
     KnnList l{0x7fffffff, 0x7fffffff};
+    int held = 0;                  // candidates in buf, all before (bD, bI) when they came
     for (int k = 0; k < 8; k++) {
         const int t = __shfl_sync(FULL, best.I, k);
         if (t == 0x7fffffff) break;
@@ -448,9 +472,11 @@ __global__ void __launch_bounds__(128)
         int idx[4];
 #pragma unroll
         for (int j = 0; j < 4; j++) {
-            const int o = min(t * kTcRows + 32 * j + lane, ncand - 1);
-            const int cy = o / Wc, cx = o - cy * Wc;
-            idx[j] = cy * stride * W + cx * stride;
+            idx[j] = min(t * kTcRows + 32 * j + lane, ncand - 1);
+            if (stride > 1) {
+                const int cy = idx[j] / Wc, cx = idx[j] - cy * Wc;
+                idx[j] = cy * stride * W + cx * stride;
+            }
 #pragma unroll
             for (int v = 0; v < NV; v++)
                 r[j][v] = __ldg(reinterpret_cast<const uint4 *>(fc + (size_t)idx[j] * P) + v);
@@ -465,10 +491,29 @@ __global__ void __launch_bounds__(128)
                 nn = __dp4a((int)cw, (int)cw, nn);
             }
             const int d = nn + qn - 2 * dot;
-            const bool real = t * kTcRows + 32 * j + lane < ncand;
-            knn_take(l, real ? d : 0x7fffffff, idx[j], lane, bD, 0x7fffffff);
+            const bool hit = t * kTcRows + 32 * j + lane < ncand && lex_less(d, idx[j], bD, bI);
+            const unsigned m = __ballot_sync(FULL, hit);
+            if (!m) continue;
+            if (held + __popc(m) > 32) {   // full: into the list, which lowers the bound
+                __syncwarp();
+                const int2 e = lane < held ? buf[lane] : make_int2(0x7fffffff, 0x7fffffff);
+                knn_take(l, e.x, e.y, lane, bD, bI);
+                knn_take(l, hit ? d : 0x7fffffff, idx[j], lane, bD, bI);
+                held = 0;
+                const int D = __shfl_sync(FULL, l.D, 7), I = __shfl_sync(FULL, l.I, 7);
+                if (lex_less(D, I, bD, bI)) bD = D, bI = I;
+            } else {
+                if (hit) buf[held + __popc(m & ((1u << lane) - 1))] = make_int2(d, idx[j]);
+                held += __popc(m);
+            }
         }
     }
+    __syncwarp();
+    const int2 e = lane < held ? buf[lane] : make_int2(0x7fffffff, 0x7fffffff);
+    if (__any_sync(FULL, l.D != 0x7fffffff))
+        knn_take(l, e.x, e.y, lane, bD, bI);
+    else
+        l = knn_sort(e.x, e.y, buf, lane);
     knn_finish<C>(out, q, lane, l);
 }
 
