@@ -308,6 +308,7 @@ __global__ void k_upsample(const uint32_t *__restrict__ pflow, int WP, const uin
 }
 
 #include "ff_sweep.cuh"
+#include "ff_block.cuh"
 #include "ff_peaks.cuh"
 #include "ff_wht_tc.cuh"
 
@@ -595,7 +596,7 @@ ff_status check_cuda(ff_ctx *ctx, cudaError_t e, const char *what) {
 const char *const kKernelNames[] = {"k_features", "k_seed_prep", "k_seed_scan", "k_seed_merge",
                                     "k_seed_rerank", "k_seed_given", "k_upsample",
                                     "k_sweep", "k_export", "k_filter", "k_dense", "k_region",
-                                    "k_sparsify"};
+                                    "k_sparsify", "k_search"};
 constexpr int kNumKernels = sizeof(kKernelNames) / sizeof(kKernelNames[0]);
 
 int kernel_id(const char *name) {
@@ -868,6 +869,53 @@ int search_radius(const ff_config &cfg, int L, int t) {
     return (plus_level(cfg, L) && t < 4) ? 2 * cfg.radius_q3 : cfg.radius_q3;
 }
 
+SearchArgs search_args(const ff_ctx *c, int d, int L, int t, uint32_t pair_id) {
+    return SearchArgs{t, d, search_radius(c->cfg, L, t), c->cfg.seed, pair_id};
+}
+
+// One sweep by blocks of columns; it also does the random search of the sweep
+// before it, where there is one.
+template <int C>
+ff_status launch_sweep_block(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L,
+                             uint32_t *flow, int *cost, int W, int H, int L, int t,
+                             uint32_t pair_id) {
+    DirState &st = c->dir[d];
+    BlockArgs a;
+    a.f1L = f1L;
+    a.f2L = f2L;
+    a.flow = flow;
+    a.cost = cost;
+    a.edge = st.edge;
+    a.ticket = st.ticket + (size_t)L * kMaxIters + t;
+    a.err = st.err;
+    a.W = W;
+    a.H = H;
+    a.L = L;
+    level_dims(W, H, L, &a.U, &a.V);
+    a.d = t & 3;
+    a.search = t > 0 && search_after(c->cfg, L, t - 1) ? 1 : 0;
+    a.rs = search_args(c, d, L, t - 1, pair_id);
+    a.epoch = 1u + (uint32_t)(L * kMaxIters + t);
+    a.wait_ns = c->wait_ns;
+    a.force_timeout = c->force_timeout;
+    const int per = kBlkRows * kBlkCluster, clusters = (a.V + per - 1) / per;
+    prof_begin(c, "k_sweep");
+    k_sweep_block<C><<<clusters * kBlkCluster, kBlkThreads, block_smem_bytes(a.U), c->stream>>>(a);
+    return check_launch(c, "k_sweep");
+}
+
+// the random search after sweep t, where no further sweep follows to do it
+template <int C>
+ff_status launch_search(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L, uint32_t *flow,
+                        int *cost, int W, int H, int L, int t, uint32_t pair_id) {
+    int U, V;
+    level_dims(W, H, L, &U, &V);
+    prof_begin(c, "k_search");
+    k_search<C><<<(U * V + 127) / 128, 128, 0, c->stream>>>(search_args(c, d, L, t, pair_id), f1L,
+                                                            f2L, W, H, L, U, V, flow, cost);
+    return check_launch(c, "k_search");
+}
+
 ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L, uint32_t *flow,
                        int *cost, int W, int H, int L, int t, uint32_t pair_id) {
     DirState &st = c->dir[d];
@@ -1003,8 +1051,20 @@ ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seed
         }
         if (s) return s;
         const int sweeps = (L == until_level) ? until_sweeps : level_sweeps(c->cfg, L);
+        const bool rows = c->sweep_lanes == 4;
         for (int t = 0; t < sweeps; t++) {
-            s = launch_sweep(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
+            if (!rows)
+                s = launch_sweep(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
+            else if (c->C == 1)
+                s = launch_sweep_block<1>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
+            else
+                s = launch_sweep_block<3>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
+            if (s) return s;
+        }
+        if (rows && sweeps > 0 && search_after(c->cfg, L, sweeps - 1)) {
+            s = c->C == 1
+                    ? launch_search<1>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id)
+                    : launch_search<3>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id);
             if (s) return s;
         }
         WP = WL;
@@ -1254,11 +1314,15 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
     int ndev = 0;
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return FF_ECUDA;
     DeviceGuard guard(device);
-    // the seeding's candidate ring takes more than 48 KB of shared memory
+    // these take more than 48 KB of shared memory (the sweep: on wide frames)
     if (cudaFuncSetAttribute(k_seed_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc_seed_smem_bytes<1>()) != cudaSuccess ||
         cudaFuncSetAttribute(k_seed_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             tc_seed_smem_bytes<2>()) != cudaSuccess) {
+                             tc_seed_smem_bytes<2>()) != cudaSuccess ||
+        cudaFuncSetAttribute(k_sweep_block<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)block_smem_bytes(FF_MAX_DIM)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_sweep_block<3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)block_smem_bytes(FF_MAX_DIM)) != cudaSuccess) {
         cudaGetLastError();
         return FF_ECUDA;
     }

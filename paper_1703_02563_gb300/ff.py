@@ -350,7 +350,7 @@ def ff_kernel_stats(ctx: int, kernel: str) -> tuple[int, float]:
 
 KERNELS = ("k_features", "k_seed_prep", "k_seed_scan", "k_seed_merge", "k_seed_rerank", "k_seed_given",
            "k_upsample", "k_sweep", "k_export", "k_filter", "k_dense", "k_region",
-           "k_sparsify")
+           "k_sparsify", "k_search")
 
 
 def ff_launch_count(ctx: int) -> int:
