@@ -216,6 +216,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
     k_sweep_block(const BlockArgs a) {
     constexpr int P = Geo<C>::P, LW = P / 8;   // bytes per vector; words of an evaluating lane
     constexpr unsigned FULL = 0xffffffffu;
+    constexpr bool kEarly = C == 3;
     extern __shared__ __align__(16) unsigned long long vin_all[];   // [kBlkRows][4 NB]
     __shared__ __align__(16) BlockShared sm;
     volatile int *v_abort = &sm.abort;
@@ -295,6 +296,39 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
             const uint32_t lo = __byte_perm((uint32_t)lx, (uint32_t)loy, 0x5410);
             const uint32_t hi = __byte_perm((uint32_t)(lx + 8 * (W - 1)), (uint32_t)hiy, 0x5410);
             const uint32_t slot = stage + (uint32_t)(b & (kBlkRing - 1)) * (uint32_t)sizeof(BlockStage);
+            // What needs no neighbour: the staged block, the windows of the four columns, the
+            // query.  For Lab frames before the wait, where it costs the rows below nothing;
+            // for gray ones, whose evaluations are short, in the shadow of the tap loads
+            // (the 1024x436 Lab pair 8.28 -> 8.00 ms, the 1242x375 gray one 5.81 against
+            // 6.47 ms the other way round).
+            uint4 cf, cc, ca, cb;
+            uint32_t lo1, hi1, lo2, hi2, lo3, hi3;
+            int4 seed[LW];
+            auto own_part = [&]() -> bool {
+                cb = lds128s(slot + 48);
+                // not staged yet?  (A vote: a 16-byte load is served in parts, so the lanes
+                // need not see the same tag.)
+                if (!__all_sync(FULL, cb.z == (uint32_t)b + 1)) {
+                    unsigned long long t0 = 0;
+                    for (int k = 1;; k++) {
+                        cb = lds128s(slot + 48);
+                        if (__all_sync(FULL, cb.z == (uint32_t)b + 1)) break;
+                        if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return false;
+                    }
+                }
+                cf = lds128s(slot), cc = lds128s(slot + 16), ca = lds128s(slot + 32);
+                lo1 = add_s16x2(lo0, wstep), hi1 = add_s16x2(hi0, wstep);
+                lo2 = add_s16x2(lo1, wstep), hi2 = add_s16x2(hi1, wstep);
+                lo3 = add_s16x2(lo2, wstep), hi3 = add_s16x2(hi2, wstep);
+#pragma unroll
+                for (int k = 0; k < LW; k++) seed[k] = query_seed(qn.w[k]);
+                const int u = min((b + 1) * kBlkCols + tgt, U - 1);
+                qn = ldg_words<LW>(qrow + (uint32_t)(flipx ? U - 1 - u : u) * P);
+                return true;
+            };
+            if constexpr (kEarly) {
+                if (!own_part()) goto finished;
+            }
             // the values above
             unsigned long long va = 0;
             if (has_v) {
@@ -317,31 +351,10 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
             const Words<LW> tc = ldg_words<LW>(f2L + (o00 + dy)),
                             td = ldg_words<LW>(f2L + (o00 + dx + dy));
             const uint32_t w = (uint32_t)(8 + 255 * (sx & 7)) * (uint32_t)(8 + 65535 * (sy & 7));
-            // while they load: the staged block, the values above, the windows of the
-            // four columns, the query
-            uint4 cb = lds128s(slot + 48);
-            // not staged yet?  (A vote: a 16-byte load is served in parts, so the lanes
-            // need not see the same tag.)
-            if (!__all_sync(FULL, cb.z == (uint32_t)b + 1)) {
-                unsigned long long t0 = 0;
-                for (int k = 1;; k++) {
-                    cb = lds128s(slot + 48);
-                    if (__all_sync(FULL, cb.z == (uint32_t)b + 1)) break;
-                    if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) goto finished;
-                }
+            if constexpr (!kEarly) {
+                if (!own_part()) goto finished;
             }
-            const uint4 cf = lds128s(slot), cc = lds128s(slot + 16), ca = lds128s(slot + 32);
             const uint4 vf0 = lds128s(vin), vf1 = lds128s(vin + 16);
-            const uint32_t lo1 = add_s16x2(lo0, wstep), hi1 = add_s16x2(hi0, wstep);
-            const uint32_t lo2 = add_s16x2(lo1, wstep), hi2 = add_s16x2(hi1, wstep);
-            const uint32_t lo3 = add_s16x2(lo2, wstep), hi3 = add_s16x2(hi2, wstep);
-            int4 seed[LW];
-#pragma unroll
-            for (int k = 0; k < LW; k++) seed[k] = query_seed(qn.w[k]);
-            {
-                const int u = min((b + 1) * kBlkCols + tgt, U - 1);
-                qn = ldg_words<LW>(qrow + (uint32_t)(flipx ? U - 1 - u : u) * P);
-            }
             uint32_t acc0 = 0, acc1 = 0;
 #pragma unroll
             for (int k = 0; k < LW; k += 2) {

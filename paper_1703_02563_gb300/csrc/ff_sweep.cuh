@@ -456,10 +456,10 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
             const int j = i + A;
             if (j < NS && ocons <= j - DI) {
                 unsigned long long t0 = 0;
-                while (true) {
+                for (int k = 1;; k++) {
                     ocons = *v_out_cons;
                     if (__all_sync(FULL, ocons > j - DI)) break;
-                    if (wait_expired(t0, a.wait_ns, v_abort, a.err)) {
+                    if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) {
                         cp_async_wait<0>();
                         return;
                     }
@@ -504,11 +504,11 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
             const unsigned long long *oslot = &sm.out[i & (DO - 1)][k];
             unsigned long long e;
             unsigned long long t0 = 0;
-            while (true) {
+            for (int k = 1;; k++) {
                 e = lds64(oslot);
                 const bool ok = (uint32_t)(e >> 52) == (uint32_t)(i & 0xFFF);
                 if (__all_sync(FULL, ok)) break;
-                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+                if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
             }
             constexpr int HLW = SG::HL_;
             const int gw = g < HLW ? g : 0;              // lanes past the words evaluate nothing
@@ -591,8 +591,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
         if (need_top) ok = ok && (uint32_t)(te >> 32) == (uint32_t)(i + 1);
         if (!__all_sync(FULL, ok)) {
             unsigned long long t0 = 0;
-            while (true) {
-                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+            for (int k = 1;; k++) {
+                if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
                 ready = *v_in_ready;
                 ocons = *v_out_cons;
                 ok = ready > i && ocons > i - DO;
