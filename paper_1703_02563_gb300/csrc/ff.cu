@@ -545,7 +545,7 @@ struct ff_ctx {
     int *rf_parent = nullptr, *rf_size = nullptr;
     uint8_t *rf_flag = nullptr;
     unsigned long long wait_ns = 2000000000ull;
-    int sweep_lanes = 4;   // propagation-warp lanes per grid point in the sweep: 2, 4 or 8
+    int sweep_lanes = 4;   // 2: the sweep for many pairs in flight; 4 (or 8): for one pair
     int force_timeout = 0;
     long long launches = 0;
     std::string last_error;
@@ -696,11 +696,10 @@ size_t level_offset(int W, int H, int P, int L) {
     return off;
 }
 
-// rows of one sweep strip for `lanes` propagation-warp lanes per grid point
-// (8 gives the smallest strips)
-int rows_per_strip(int lanes) {
-    return lanes == 2 ? SweepGeo<1, 1>::RW : (lanes == 8 ? SweepGeo<1, 4>::RW : SweepGeo<1, 2>::RW);
-}
+// rows between the boundary rows that either sweep kernel keeps: strips of
+// k_sweep_many, clusters of k_sweep_block
+constexpr int kEdgeRows = SweepGeo<1>::RW;
+static_assert(kEdgeRows <= kBlkRows * kBlkCluster, "boundary rows");
 
 template <typename T>
 cudaError_t alloc(T **p, size_t count) {
@@ -900,7 +899,20 @@ ff_status launch_sweep_block(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t
     a.force_timeout = c->force_timeout;
     const int per = kBlkRows * kBlkCluster, clusters = (a.V + per - 1) / per;
     prof_begin(c, "k_sweep");
-    k_sweep_block<C><<<clusters * kBlkCluster, kBlkThreads, block_smem_bytes(a.U), c->stream>>>(a);
+    // a sweep after another starts up while that one ends (see the kernel), on
+    // levels whose CTAs leave room for it
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(clusters * kBlkCluster);
+    cfg.blockDim = dim3(blk_threads(C));
+    cfg.dynamicSmemBytes = block_smem_bytes(a.U);
+    cfg.stream = c->stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = t > 0 && a.U <= kBlkOverlap ? 1 : 0;
+    const ff_status s = check_cuda(c, cudaLaunchKernelEx(&cfg, k_sweep_block<C>, a), "k_sweep");
+    if (s) return s;
     return check_launch(c, "k_sweep");
 }
 
@@ -947,23 +959,12 @@ ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L,
     a.epoch = 1u + (uint32_t)(L * kMaxIters + t);
     a.wait_ns = c->wait_ns;
     a.force_timeout = c->force_timeout;
-    const int R = rows_per_strip(c->sweep_lanes);
-    const int nstrips = (HL + R - 1) / R;
+    const int nstrips = (HL + SweepGeo<1>::RW - 1) / SweepGeo<1>::RW;
     prof_begin(c, "k_sweep");
-#define FF_LAUNCH_SWEEP(CC, LPC) \
-    k_sweep<CC, LPC><<<nstrips, SweepGeo<CC, LPC>::THREADS, 0, c->stream>>>(a)
-    if (c->C == 1) {
-        if (c->sweep_lanes == 2)
-            k_sweep_many<1><<<nstrips, SweepGeo<1, 1>::THREADS, 0, c->stream>>>(a);
-        else if (c->sweep_lanes == 8) FF_LAUNCH_SWEEP(1, 4);
-        else FF_LAUNCH_SWEEP(1, 2);
-    } else {
-        if (c->sweep_lanes == 2)
-            k_sweep_many<3><<<nstrips, SweepGeo<3, 1>::THREADS, 0, c->stream>>>(a);
-        else if (c->sweep_lanes == 8) FF_LAUNCH_SWEEP(3, 4);
-        else FF_LAUNCH_SWEEP(3, 2);
-    }
-#undef FF_LAUNCH_SWEEP
+    if (c->C == 1)
+        k_sweep_many<1><<<nstrips, SweepGeo<1>::THREADS, 0, c->stream>>>(a);
+    else
+        k_sweep_many<3><<<nstrips, SweepGeo<3>::THREADS, 0, c->stream>>>(a);
     return check_launch(c, "k_sweep");
 }
 
@@ -1051,9 +1052,9 @@ ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seed
         }
         if (s) return s;
         const int sweeps = (L == until_level) ? until_sweeps : level_sweeps(c->cfg, L);
-        const bool rows = c->sweep_lanes == 4;
+        const bool block = c->sweep_lanes != 2;
         for (int t = 0; t < sweeps; t++) {
-            if (!rows)
+            if (!block)
                 s = launch_sweep(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
             else if (c->C == 1)
                 s = launch_sweep_block<1>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
@@ -1061,7 +1062,7 @@ ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seed
                 s = launch_sweep_block<3>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
             if (s) return s;
         }
-        if (rows && sweeps > 0 && search_after(c->cfg, L, sweeps - 1)) {
+        if (block && sweeps > 0 && search_after(c->cfg, L, sweeps - 1)) {
             s = c->C == 1
                     ? launch_search<1>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id)
                     : launch_search<3>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id);
@@ -1337,7 +1338,7 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
     c->stream = (cudaStream_t)cuda_stream;
     c->C = cfg->channels;
     c->P = cfg->channels == 1 ? 16 : 32;
-    c->sweep_lanes = 4;   // the shortest step chain, for one pair at a time
+    c->sweep_lanes = 4;   // one pair at a time
     c->S = cfg->scales;
     c->I = cfg->iters;
     c->maxW = cfg->max_width;
@@ -1347,8 +1348,7 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
     level_dims(c->maxW, c->maxH, c->S - 1, &WS, &HS);
     c->nq_cap = (size_t)WS * HS;
     const size_t npix = (size_t)c->maxW * c->maxH;
-    const int R = rows_per_strip(8);   // the smallest strip
-    c->edge_cap = (size_t)((c->maxH + R - 1) / R) * c->maxW;
+    c->edge_cap = (size_t)((c->maxH + kEdgeRows - 1) / kEdgeRows) * c->maxW;
     cudaError_t e = cudaSuccess;
     for (int s = 0; s < 2 && e == cudaSuccess; s++) {
         e = alloc(&c->feat[s], c->feat_cap);
@@ -2190,8 +2190,7 @@ size_t context_bytes(const ff_config &cfg) {
     int WS, HS;
     level_dims(cfg.max_width, cfg.max_height, cfg.scales - 1, &WS, &HS);
     const size_t nq = (size_t)WS * HS, K = C == 1 ? 16 : 32, pad = kTcRows;
-    const int R = rows_per_strip(8);
-    const size_t edge = (size_t)((cfg.max_height + R - 1) / R) * cfg.max_width;
+    const size_t edge = (size_t)((cfg.max_height + kEdgeRows - 1) / kEdgeRows) * cfg.max_width;
     size_t b = 2 * level_offset(cfg.max_width, cfg.max_height, P, cfg.scales);   // features
     b += 2 * npix * C + 3 * npix * 4 + npix;                                    // staging
     b += npix * (4 + 4 + 1);                                                    // region scratch

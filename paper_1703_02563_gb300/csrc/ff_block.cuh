@@ -99,9 +99,16 @@ __global__ void __launch_bounds__(128)
 constexpr int kBlkCols = 4;                  // columns decided per step
 constexpr int kBlkRows = 4;                  // rows of a strip, one warp each
 constexpr int kBlkCluster = 8;               // strips of a cluster
-constexpr int kBlkStagers = 4;               // stager warps
+// Stager warps: Lab blocks take four (with two a 1024x436 pair 8.19 -> 8.52 ms), gray
+// ones two (with four a 1242x375 pair 5.26 -> 5.55 ms: more of them only contend with
+// the rows for issue slots).
+__host__ __device__ constexpr int blk_stagers(int C) { return C == 3 ? 4 : 2; }
+__host__ __device__ constexpr int blk_threads(int C) { return (kBlkRows + blk_stagers(C) + 1) * 32; }
 constexpr int kBlkRing = 16;                 // staged blocks per row
-constexpr int kBlkThreads = (kBlkRows + kBlkStagers + 1) * 32;
+// Levels up to this wide start the next sweep's launch early: its waiting CTAs hold
+// room on the SMs (a 128x96 pair 973 -> 917 us, 1024x436 8.53 -> 8.45 ms; on every
+// level the latter took 8.60 ms).
+constexpr int kBlkOverlap = 512;
 constexpr uint32_t kBlkNone = 0x80000000u;   // cost of a candidate that does not exist
 
 struct BlockArgs {
@@ -194,6 +201,9 @@ __device__ __forceinline__ uint4 lds128s(uint32_t p) {
 __device__ __forceinline__ void sts32s(uint32_t p, uint32_t v) {
     asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
+__device__ __forceinline__ void launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 // packed 16-bit add (no carry between the halves)
 __device__ __forceinline__ uint32_t add_s16x2(uint32_t a, uint32_t b) {
     uint32_t r;
@@ -212,11 +222,12 @@ __host__ __device__ constexpr size_t block_smem_bytes(int U) {
 }
 
 template <int C>
-__global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThreads)
+__global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_threads(C))
     k_sweep_block(const BlockArgs a) {
     constexpr int P = Geo<C>::P, LW = P / 8;   // bytes per vector; words of an evaluating lane
     constexpr unsigned FULL = 0xffffffffu;
     constexpr bool kEarly = C == 3;
+    constexpr int kStagers = blk_stagers(C), kThreads = blk_threads(C);
     extern __shared__ __align__(16) unsigned long long vin_all[];   // [kBlkRows][4 NB]
     __shared__ __align__(16) BlockShared sm;
     volatile int *v_abort = &sm.abort;
@@ -225,12 +236,15 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
     const int U = a.U, V = a.V, W = a.W, H = a.H, L = a.L, n = 1 << L, half = n >> 1;
     const int NB = (U + kBlkCols - 1) / kBlkCols, UP = NB * kBlkCols;
     const uint32_t rank = cluster_rank();
-    for (int j = tid; j < kBlkRows * UP; j += kBlkThreads) vin_all[j] = 0ull;
-    for (int j = tid; j < kBlkRows * kBlkRing; j += kBlkThreads) (&sm.stage[0][0])[j].tag = 0;
+    for (int j = tid; j < kBlkRows * UP; j += kThreads) vin_all[j] = 0ull;
+    for (int j = tid; j < kBlkRows * kBlkRing; j += kThreads) (&sm.stage[0][0])[j].tag = 0;
     if (tid < kBlkRows) sm.done[tid] = 0;
     if (tid == 0) sm.abort = 0;
     if (rank == 0 && tid == 0) sm.cluster = (int)atomicAdd(a.ticket, 1u);
     cluster_sync();   // (also: every CTA has started and cleared its rows)
+    // Up to here nothing of the sweep before is touched: the launch may overlap its
+    // end (programmatic dependent launch).
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int cluster = (int)ld_cluster_u32(mapa(smem_addr(&sm.cluster), 0));
     const int strip = cluster * kBlkCluster + (int)rank;
     const int v0 = strip * kBlkRows;
@@ -239,6 +253,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
 
     if (v0 >= V) {
         // no rows here
+        launch_dependents();
     } else if (warp < kBlkRows) {
         // ================= a row =================
         const int v = v0 + warp;
@@ -417,7 +432,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
         }
         // rows past the frame's edge never hold a stager back
         if (!live && lane == 0) sts32s(done, NB + kBlkRing);
-    } else if (warp < kBlkRows + kBlkStagers) {
+    } else if (warp < kBlkRows + kStagers) {
         // ================= a stager =================
         // pass p: blocks 2 p and 2 p + 1 of the four rows, one point per lane
         const int w = warp - kBlkRows;
@@ -426,15 +441,17 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(kBlkThread
         const int gy = flipy ? V - 1 - v : v;
         const int py = gy * n;
         const int loy = -8 * py, hiy = 8 * (H - 1) - 8 * py;
-        for (int p = w; 2 * p < NB; p += kBlkStagers) {
+        for (int p = w; 2 * p < NB; p += kStagers) {
             // room: every row is past the block that used the slots before
             unsigned long long t0 = 0;
             for (int k = 1;; k++) {
+                if (k > 1) __nanosleep(200);
                 const bool ok = lane >= kBlkRows ||
                                 (int)lds32s(smem_addr(&sm.done[lane])) + kBlkRing >= 2 * p + 2;
                 if (__all_sync(FULL, ok)) break;
                 if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) goto finished;
             }
+            if (p == 0) launch_dependents();   // (the next sweep's launch may come in)
             const int u = 8 * p + (lane & 7);
             const bool in = v < V && u < U;
             uint32_t f = kFlowInvalid, c = 0x7fffffffu;

@@ -20,65 +20,48 @@ struct SweepArgs {
     int force_timeout;
 };
 
-// Geometry of a sweep CTA.  A CTA owns a strip of RW rows and has five warps:
-// propagation (warp 0), random search (1), input stager (2), L1 warmer (3)
-// and boundary-row loader (4), so the propagation warp shares its SM
-// sub-partition only with the loader, which mostly sleeps.  The layout for
-// many pairs in flight (LPC = 1) has no warmer (the loader is warp 3): with
-// several CTAs per SM the warming copies cost more issue slots than the L1
-// hits they buy (measured on the 32- and 64-pair batches).
+// Geometry of a sweep CTA of the layout for many pairs in flight (batch and
+// server slots; one pair at a time runs ff_block.cuh).  A CTA owns a strip of RW
+// rows and has four warps: propagation (warp 0), random search (1), input stager
+// (2) and boundary-row loader (3).
 //
-// A grid point is handled by G = 2 LPC lanes of the propagation warp: lanes
-// 0..LPC-1 evaluate the vertical candidate, lanes LPC..2 LPC-1 the horizontal
-// one, each over WPC of the NWU feature words (4 dimensions each) that hold
-// codes (7 for Lab, 3 for gray; the rest of the P bytes is zero on both
-// sides, so a lane may include a padding word: it adds |0 - 0| = 0).
-template <int C, int LPC> struct SweepGeo {
+// A grid point is handled by G = 2 lanes of the propagation warp, one per
+// candidate (0: vertical, 1: horizontal), each over the NWU feature words (4
+// dimensions each) that hold codes (7 for Lab, 3 for gray; the rest of the P
+// bytes is zero on both sides).
+template <int C> struct SweepGeo {
     static constexpr int P = Geo<C>::P;              // bytes per feature vector: 16, 32
     static constexpr int NW = P / 4;                 // words per feature vector: 4, 8
     static constexpr int NWU = C == 3 ? 7 : 3;       // words holding codes
-    static constexpr int G = 2 * LPC;                // lanes per grid point
+    static constexpr int G = 2;                      // lanes per grid point
     static constexpr int RW = 32 / G;                // rows per strip
-    static constexpr int WPC = (NWU + LPC - 1) / LPC;              // words per lane and candidate
-    static constexpr int LWP = WPC <= 1 ? 1 : (WPC <= 2 ? 2 : (WPC <= 4 ? 4 : 8));  // words loaded
-    static_assert(LPC * LWP <= NW || LPC == 1, "lane words");
-    static constexpr int WPH = NW >= G ? NW / G : 1; // words per lane in the random search
-    static constexpr int HL_ = NW / WPH;             // random-search lanes holding words
-    static constexpr int QB = P / G >= 4 ? P / G : 4;  // query bytes a stager lane copies
-    static constexpr int QL = P / QB;                // stager lanes holding query bytes
-    // One lane per candidate is the layout for many pairs in flight: a
-    // shorter input ring (8 steps, staged 4 ahead) and a register bound let
-    // six CTAs share an SM, whose other CTAs hide the staging latency.
-    static constexpr int DI = LPC == 1 ? 8 : 16;     // staged-input ring depth (steps)
+    static constexpr int LWP = NW;                   // words loaded by a lane
+    static constexpr int WPH = NW / G;               // words per lane in the random search
+    static constexpr int QB = P / G;                 // query bytes a stager lane copies
+    // A short input ring (8 steps, staged 4 ahead) and a register bound let eight CTAs
+    // share an SM, whose other CTAs hide the staging latency.
+    static constexpr int DI = 8;                     // staged-input ring depth (steps)
     static constexpr int DO = 16;                    // result ring depth (steps)
-    static constexpr int A = LPC == 1 ? 4 : 8;       // staging distance (steps ahead)
-    static constexpr int MIN_CTAS = 8;               // CTAs per SM the registers allow (LPC 1)
-    static constexpr bool WARM = LPC != 1;           // an L1-warming warp
-    static constexpr int LOADER = WARM ? 4 : 3;      // the loader's warp
+    static constexpr int A = 4;                      // staging distance (steps ahead)
+    static constexpr int MIN_CTAS = 8;               // CTAs per SM the registers allow
+    static constexpr int LOADER = 3;                 // the loader's warp
     static constexpr int LRING = 128;                // previous strip -> this strip ring
     static constexpr int NB = 8 / G;                 // random-search offsets per lane per 8 steps
-    static constexpr int PD = 1;                     // L1 warming distance (level pixels)
-    static constexpr int PF_COLS = 4;                // feature columns warmed from the target on
-    static constexpr int PF_ROWS = LPC == 2 ? 6 : 4; // feature rows warmed around the target
-    // Lab: the staged pre-sweep flow of the point PDS steps ahead is warmed too
-    // (1.7% faster on the Sintel-shaped pair; on gray frames it cost 10%)
-    static constexpr int PDS = C == 3 ? 6 : 0;
-    static constexpr int THREADS = (WARM ? 5 : 4) * 32;
+    static constexpr int THREADS = 4 * 32;
 };
 
-template <int C, int LPC> struct SweepShared {
-    using SG = SweepGeo<C, LPC>;
-    // -64 x query, per word (4 dimensions).  The batch layout's rows are
-    // padded by one word so that its 16 rows' loads spread over the banks
-    // (6.7% faster on the Sintel-shaped pair; neutral for the one-pair layouts)
-    int4 in_nq[SG::DI][SG::RW][SG::NW + (LPC == 1 ? 1 : 0)];
+template <int C> struct SweepShared {
+    using SG = SweepGeo<C>;
+    // -64 x query, per word (4 dimensions).  The rows are padded by one word so
+    // that the 16 rows' loads spread over the banks (the 32- and 64-pair batches
+    // ran 4% and 3% faster)
+    int4 in_nq[SG::DI][SG::RW][SG::NW + 1];
     uint8_t in_raw[SG::DI][SG::RW][SG::P];        // query bytes as copied
     uint32_t in_flow[SG::DI][SG::RW];
     int in_cost[SG::DI][SG::RW];
     unsigned long long out[SG::DO][SG::RW];       // (tag:12 | cost:20) << 32 | flow
     unsigned long long lring[SG::LRING];          // (column + 1) << 32 | flow
     int in_ready, out_cons, lcons, abort, strip;
-    uint32_t pf_sink[32];                         // destination of L1-warming copies
 };
 
 __device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
@@ -196,13 +179,6 @@ __device__ __forceinline__ unsigned long long pack_out(int tag, int cost, uint32
     return ((unsigned long long)(((uint32_t)(tag & 0xFFF) << 20) | c) << 32) | flow;
 }
 
-// target (1/8 px) of flow f at grid point (px, py), clamped into the frame
-__device__ __forceinline__ void target_of(uint32_t f, int px, int py, int W, int H, int &tx,
-                                          int &ty) {
-    tx = clampi(8 * px + flow_x(f), 0, 8 * (W - 1));
-    ty = clampi(8 * py + flow_y(f), 0, 8 * (H - 1));
-}
-
 // Slow path of a warp-uniform wait: returns true when the warp must give up
 // (the CTA's abort flag is up, or nothing changed for wait_ns, in which case
 // the error word gets FF_ETIMEOUT and the abort flag is raised).  t0 == 0
@@ -248,25 +224,23 @@ __device__ __forceinline__ bool wait_expired(unsigned long long &t0, unsigned lo
 //    point's offset (Philox4x32-10, counter (y*W + x, t, L, dir), key (seed,
 //    pair_id)), keeps it only if strictly better, and writes the final flow
 //    and cost.  Neighbours in this sweep see only the sweep value.
-//  * Warming warp: follows the result slots and pulls into L1 the feature
-//    sectors around each decided flow's target two points further on, where
-//    the row's next loads most likely fall (for Lab frames also those of the
-//    staged pre-sweep flows a few steps ahead).
 //  * Loader warp: copies the previous strip's boundary row into the ring.
 // Strips are handed out by a ticket counter, so a strip only waits on a
 // strip that is already running.  Every wait is bounded and warp-uniform: a
 // warp that sees no progress for wait_ns sets the error word to FF_ETIMEOUT,
 // raises the CTA's abort flag and returns; every other wait in the CTA
 // checks that flag on its slow path.
-template <int C, int LPC>
-__device__ __forceinline__ void sweep_body(const SweepArgs &a) {
-    using SG = SweepGeo<C, LPC>;
+//
+// Bounded to the registers that let MIN_CTAS CTAs share an SM.
+template <int C>
+__global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
+    k_sweep_many(const SweepArgs a) {
+    using SG = SweepGeo<C>;
     constexpr int P = SG::P, G = SG::G, RW = SG::RW;
     constexpr int DI = SG::DI, DO = SG::DO, A = SG::A, LRING = SG::LRING;
-    constexpr int WPC = SG::WPC, LWP = SG::LWP, WPH = SG::WPH, NB = SG::NB;
-    constexpr int PD = SG::PD, PF_ROWS = SG::PF_ROWS, PF_COLS = SG::PF_COLS;
+    constexpr int NWU = SG::NWU, LWP = SG::LWP, WPH = SG::WPH, NB = SG::NB;
     constexpr unsigned FULL = 0xffffffffu;
-    __shared__ __align__(16) SweepShared<C, LPC> sm;
+    __shared__ __align__(16) SweepShared<C> sm;
     volatile int *v_in_ready = &sm.in_ready;
     volatile int *v_out_cons = &sm.out_cons;
     volatile int *v_lcons = &sm.lcons;
@@ -343,81 +317,12 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
     const uint8_t *f1L = a.f1L, *f2L = a.f2L;
     const size_t rowbase = (size_t)gy * U;
 
-    if (SG::WARM && warp == 3) {
-        // ================= warming warp =================
-        // Warms L1 with the feature sectors the propagation warp will read two
-        // points after each decision: rows iy-2 .. iy+3 around the target of
-        // the decided flow at that point, columns ix .. ix+PF_COLS-1, one
-        // sector (one point's feature vector) each, by asynchronous 4-byte
-        // copies into a scratch word.  It follows the tagged result slots,
-        // so the propagation warp spends no instruction on it; a slot holding
-        // a later step than expected (this warp fell a ring behind) is taken
-        // as it is.  For Lab frames it also warms, PDS steps ahead, the 3 x 3
-        // sectors around the target of a point's staged pre-sweep flow at the
-        // next point: in a settled field that flow is the likely value of the
-        // next point's horizontal source and of the point below's vertical one.
-        const int sxdir = flipx ? -1 : 1;
-        int i = 0, wready = 0;
-        unsigned long long t0 = 0;
-        while (i < NS) {
-            const unsigned long long e = lds64(&sm.out[i & (DO - 1)][k]);
-            const uint32_t dd = ((uint32_t)(e >> 52) - (uint32_t)i) & 0xFFFu;   // its step - i
-            if (!__all_sync(FULL, dd < 0x800u)) {
-                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) break;
-                continue;
-            }
-            t0 = 0;
-            const int u = i + (int)dd - k;                // the point decided in that step
-            const uint32_t f = (uint32_t)e;
-            if (row_ok && u >= 0 && u < U && f != kFlowInvalid) {
-                const int gx = flipx ? U - 1 - u : u;
-                int tx, ty;
-                target_of(f, (gx + sxdir * (PD + 1)) * n, py, W, H, tx, ty);
-                const int ix = min((tx + half) >> (L + 3), U - 1);
-                const int iy0 = ((ty + half) >> (L + 3)) - (PF_ROWS / 2 - 1);
-#pragma unroll
-                for (int rr = 0; rr < (PF_ROWS + G - 1) / G; rr++) {
-                    const int row = g + rr * G;
-                    if (row < PF_ROWS) {
-                        const uint8_t *rowp = f2L + (size_t)clampi(iy0 + row, 0, V - 1) * U * P;
-#pragma unroll
-                        for (int cc = 0; cc < PF_COLS; cc++)
-                            cp_async4(&sm.pf_sink[lane], rowp + (size_t)min(ix + cc, U - 1) * P);
-                    }
-                }
-            }
-            if (SG::PDS > 0) {
-                const int j = i + (int)dd + SG::PDS;
-                if (wready <= j) wready = *v_in_ready;
-                const int uj = j - k;
-                if (j < wready && row_ok && uj >= 0 && uj + 1 < U && g < 3) {
-                    const uint32_t fj = ((volatile uint32_t *)sm.in_flow[j & (DI - 1)])[k];
-                    if (fj != kFlowInvalid) {
-                        const int gxn = flipx ? U - 1 - (uj + 1) : uj + 1;
-                        int tx, ty;
-                        target_of(fj, gxn * n, py, W, H, tx, ty);
-                        const int ixn = tx >> (L + 3), iyn = (ty >> (L + 3)) + g;
-                        const uint8_t *rowp = f2L + (size_t)clampi(iyn, 0, V - 1) * U * P;
-#pragma unroll
-                        for (int cc = -1; cc <= 1; cc++)
-                            cp_async4(&sm.pf_sink[lane],
-                                      rowp + (size_t)clampi(ixn + cc, 0, U - 1) * P);
-                    }
-                }
-            }
-            i += 1 + (int)__reduce_min_sync(FULL, dd);
-        }
-        cp_async_commit();
-        cp_async_wait<0>();
-        return;
-    }
-
     if (warp == 2) {
         // ================= stager warp =================
         // step j's inputs -> ring slot j mod DI: flow and cost, the query's
         // bytes (P / G per lane), then -64 q per dimension.  A slot is reused
         // only after the random-search warp (the last reader) took its step.
-        constexpr int QB = SG::QB, QL = SG::QL;            // query bytes per lane, lanes used
+        constexpr int QB = SG::QB;                         // query bytes per lane
         auto stage = [&](int j) {
             const int uj = j - k;
             if (row_ok && uj >= 0 && uj < U) {
@@ -426,17 +331,13 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
                 const int slot = j & (DI - 1);
                 if (g == 0) cp_async4(&sm.in_flow[slot][k], a.flow + pi);
                 if (g == G - 1) cp_async4(&sm.in_cost[slot][k], a.cost + pi);
-                if (g < QL) {
-                    uint8_t *dst = &sm.in_raw[slot][k][QB * g];
-                    const uint8_t *srcq = f1L + pi * P + QB * g;
-                    if constexpr (QB == 16) cp_async16ca(dst, srcq);
-                    else if constexpr (QB == 8) cp_async8(dst, srcq);
-                    else cp_async4(dst, srcq);
-                }
+                uint8_t *dst = &sm.in_raw[slot][k][QB * g];
+                const uint8_t *srcq = f1L + pi * P + QB * g;
+                if constexpr (QB == 16) cp_async16ca(dst, srcq);
+                else cp_async8(dst, srcq);
             }
         };
         auto convert = [&](int j) {
-            if (g >= QL) return;
             const int slot = j & (DI - 1);
             const uint32_t *raw = reinterpret_cast<const uint32_t *>(&sm.in_raw[slot][k][QB * g]);
 #pragma unroll
@@ -456,10 +357,10 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
             const int j = i + A;
             if (j < NS && ocons <= j - DI) {
                 unsigned long long t0 = 0;
-                for (int k = 1;; k++) {
+                while (true) {
                     ocons = *v_out_cons;
                     if (__all_sync(FULL, ocons > j - DI)) break;
-                    if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) {
+                    if (wait_expired(t0, a.wait_ns, v_abort, a.err)) {
                         cp_async_wait<0>();
                         return;
                     }
@@ -504,17 +405,15 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
             const unsigned long long *oslot = &sm.out[i & (DO - 1)][k];
             unsigned long long e;
             unsigned long long t0 = 0;
-            for (int k = 1;; k++) {
+            while (true) {
                 e = lds64(oslot);
                 const bool ok = (uint32_t)(e >> 52) == (uint32_t)(i & 0xFFF);
                 if (__all_sync(FULL, ok)) break;
-                if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
             }
-            constexpr int HLW = SG::HL_;
-            const int gw = g < HLW ? g : 0;              // lanes past the words evaluate nothing
             int4 nq[WPH];
 #pragma unroll
-            for (int j = 0; j < WPH; j++) nq[j] = lds128v(&sm.in_nq[i & (DI - 1)][k][WPH * gw + j]);
+            for (int j = 0; j < WPH; j++) nq[j] = lds128v(&sm.in_nq[i & (DI - 1)][k][WPH * g + j]);
             __syncwarp();
             if (lane == 0) *v_out_cons = i + 1;
             const uint32_t best = (uint32_t)e;
@@ -542,8 +441,7 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
                 int er = 0;
                 if (__any_sync(FULL, nR)) {
                     const TapRows t = taps_of<P>(cR, gx, gy, L, half, U, V);
-                    er = sad_taps<WPH, WPH>(f2L + 4 * WPH * gw, t, nq);
-                    if (g >= HLW) er = 0;
+                    er = sad_taps<WPH, WPH>(f2L + 4 * WPH * g, t, nq);
                 }
 #pragma unroll
                 for (int o = G / 2; o > 0; o >>= 1) er += __shfl_xor_sync(FULL, er, o);
@@ -561,11 +459,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
     }
 
     // ================= propagation warp =================
-    const int cand = g / LPC;                    // 0: vertical candidate, 1: horizontal
-    const int hw = g - cand * LPC;               // which words of the candidate
+    const int cand = g;                          // 0: vertical candidate, 1: horizontal
     const bool edge_out = (k == RW - 1) && (strip + 1 < nstrips);
     const bool top_src = v0 > 0;                 // row 0 has a row above it
-    const uint8_t *f2w = f2L + 4 * LWP * hw;     // this lane's words of every feature vector
     const int loy = -8 * py, hiy = 8 * (H - 1) - 8 * py;
     uint32_t last = kFlowInvalid;       // this row's sweep value at the previous step
     // The step has one branch besides the loop's: its inputs are checked at
@@ -591,8 +487,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
         if (need_top) ok = ok && (uint32_t)(te >> 32) == (uint32_t)(i + 1);
         if (!__all_sync(FULL, ok)) {
             unsigned long long t0 = 0;
-            for (int k = 1;; k++) {
-                if ((k & 31) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+            while (true) {
+                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
                 ready = *v_in_ready;
                 ocons = *v_out_cons;
                 ok = ready > i && ocons > i - DO;
@@ -610,9 +506,9 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
         const int scost = ((volatile int *)sm.in_cost[islot])[k];
         const uint32_t cur = active ? sflow : kFlowInvalid;
         const int ccost = active ? scost : kCostInvalid;
-        int4 nq[WPC];
+        int4 nq[NWU];
 #pragma unroll
-        for (int j = 0; j < WPC; j++) nq[j] = lds128v(&sm.in_nq[islot][k][LWP * hw + j]);
+        for (int j = 0; j < NWU; j++) nq[j] = lds128v(&sm.in_nq[islot][k][j]);
         const uint32_t vflow = (active && v > 0) ? ((k > 0) ? above : (uint32_t)te) : kFlowInvalid;
         const uint32_t hflow = (active && u > 0) ? last : kFlowInvalid;
         // both candidates clamped into the frame: 8 p + F in [0, 8(W-1)] x [0, 8(H-1)]
@@ -622,20 +518,8 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
         const uint32_t cV = clamp_s16x2(vflow, lo, hi);
         const uint32_t cH = clamp_s16x2(hflow, lo, hi);
         const TapRows t = taps_of<P>(cand == 0 ? cV : cH, gx, gy, L, half, U, V);
-        int e = sad_taps<LWP, WPC>(f2w, t, nq);
-        // this candidate's cost and the other one's (eo); with two lanes per
-        // candidate, three independent shuffles instead of two in a row
-        int eo;
-        if constexpr (LPC == 2) {
-            const int x1 = __shfl_xor_sync(FULL, e, 1), x2 = __shfl_xor_sync(FULL, e, 2),
-                      x3 = __shfl_xor_sync(FULL, e, 3);
-            e += x1;
-            eo = x2 + x3;
-        } else {
-#pragma unroll
-            for (int o = 1; o < LPC; o <<= 1) e += __shfl_xor_sync(FULL, e, o);
-            eo = __shfl_xor_sync(FULL, e, LPC);
-        }
+        const int e = sad_taps<LWP, NWU>(f2L, t, nq);
+        const int eo = __shfl_xor_sync(FULL, e, 1);   // the other candidate's
         const int ev = cand == 0 ? e : eo, eh = cand == 0 ? eo : e;
         // [current, vertical, horizontal]: lowest cost, the later one on ties
         uint32_t best = cur;
@@ -652,27 +536,13 @@ __device__ __forceinline__ void sweep_body(const SweepArgs &a) {
         // the strip's last row -> the next strip (a predicated store)
         st_relaxed_u64_if(a.edge + (size_t)strip * U + uc, ((unsigned long long)a.epoch << 32) | best,
                           edge_out && active && g == 0);
-        // result -> random-search and warming warps (tagged slot)
+        // result -> random-search warp (tagged slot)
         if (g == 0) sts64(&sm.out[i & (DO - 1)][k], pack_out(i, bcost, best));
         // the next step's inputs, read now (checked at its start)
         te_next = lds64(&sm.lring[(i + 1) & (LRING - 1)]);
         ready = *v_in_ready;
         ocons = *v_out_cons;
     }
-}
-
-// The sweep kernel.  One lane per candidate (LPC = 1) is bounded to the
-// registers that let MIN_CTAS CTAs share an SM; the other layouts run one CTA
-// per SM for a single pair, so they are compiled for one (the compiler then
-// takes 79 instead of 64 registers: 2% faster on both single-pair workloads).
-template <int C, int LPC>
-__global__ void __launch_bounds__(SweepGeo<C, LPC>::THREADS, 1) k_sweep(const SweepArgs a) {
-    sweep_body<C, LPC>(a);
-}
-template <int C>
-__global__ void __launch_bounds__(SweepGeo<C, 1>::THREADS, SweepGeo<C, 1>::MIN_CTAS)
-    k_sweep_many(const SweepArgs a) {
-    sweep_body<C, 1>(a);
 }
 
 }  // namespace ffk
