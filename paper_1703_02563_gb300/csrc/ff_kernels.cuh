@@ -88,7 +88,7 @@ __device__ __forceinline__ int sad_word(uint32_t t00, uint32_t t10, uint32_t t01
     const int e1 = __dp4a((int)__byte_perm(lo01, lo23, 0x7632), (int)w, na.y);
     const int e2 = __dp4a((int)__byte_perm(hi01, hi23, 0x5410), (int)w, na.z);
     const int e3 = __dp4a((int)__byte_perm(hi01, hi23, 0x7632), (int)w, na.w);
-    return abs(e0) + abs(e1) + abs(e2) + abs(e3);
+    return (int)(__sad(e1, 0, __sad(e0, 0, 0u)) + __sad(e3, 0, __sad(e2, 0, 0u)));
 }
 
 __device__ __forceinline__ uint32_t ldg32(const uint8_t *p) {

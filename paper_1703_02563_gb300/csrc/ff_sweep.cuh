@@ -162,10 +162,10 @@ __device__ __forceinline__ Words<NWL> ldg_words(const uint8_t *p) {
 // 64 q[d] (the query enters as the accumulator).
 template <int NWL, int NC>
 __device__ __forceinline__ int sad_taps(const uint8_t *base, const TapRows &t, const int4 *nq) {
-    const Words<NWL> a = ldg_words<NWL>(base + t.r0 + t.c0);
-    const Words<NWL> b = ldg_words<NWL>(base + t.r0 + t.c1);
-    const Words<NWL> c = ldg_words<NWL>(base + t.r1 + t.c0);
-    const Words<NWL> d = ldg_words<NWL>(base + t.r1 + t.c1);
+    const Words<NWL> a = ldg_words<NWL>(base + (uint32_t)(t.r0 + t.c0));
+    const Words<NWL> b = ldg_words<NWL>(base + (uint32_t)(t.r0 + t.c1));
+    const Words<NWL> c = ldg_words<NWL>(base + (uint32_t)(t.r1 + t.c0));
+    const Words<NWL> d = ldg_words<NWL>(base + (uint32_t)(t.r1 + t.c1));
     int e = 0;
 #pragma unroll
     for (int j = 0; j < NC; j++) e += sad_word(a.w[j], b.w[j], c.w[j], d.w[j], t.w, nq[j]);
