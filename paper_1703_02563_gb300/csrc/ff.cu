@@ -283,28 +283,36 @@ __global__ void k_seed_given(const uint32_t *__restrict__ seeds, const uint8_t *
 
 // Sec. 3.2 coarse to fine: points of level L that are points of level L+1
 // (both grid coordinates even) keep their flow, re-evaluated at scale n; the
-// other points start unset.
+// other points start unset.  blockIdx.y: which of the flows.
+struct UpsampleDir {
+    const uint32_t *pflow;
+    const uint8_t *f1L, *f2L;
+    uint32_t *flow;
+    int *cost;
+};
+struct UpsampleArgs {
+    UpsampleDir of[3];
+};
 template <int C>
-__global__ void k_upsample(const uint32_t *__restrict__ pflow, int WP, const uint8_t *f1L,
-                           const uint8_t *f2L, int W, int H, int L, int WL, int HL,
-                           uint32_t *__restrict__ flow, int *__restrict__ cost) {
+__global__ void k_upsample(const __grid_constant__ UpsampleArgs a, int WP, int W, int H, int L, int WL, int HL) {
     constexpr int P = Geo<C>::P;
+    const UpsampleDir &of = a.of[blockIdx.y];
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= WL * HL) return;
     const int gy = q / WL, gx = q - gy * WL;
     uint32_t f = kFlowInvalid;
-    if (((gx | gy) & 1) == 0) f = pflow[(gy >> 1) * WP + (gx >> 1)];
+    if (((gx | gy) & 1) == 0) f = of.pflow[(gy >> 1) * WP + (gx >> 1)];
     if (f == kFlowInvalid) {
-        flow[q] = kFlowInvalid;
-        cost[q] = kCostInvalid;
+        of.flow[q] = kFlowInvalid;
+        of.cost[q] = kCostInvalid;
         return;
     }
     uint32_t qw[P / 4];
 #pragma unroll
-    for (int w = 0; w < P / 4; w++) qw[w] = ldg32(f1L + (size_t)q * P + 4 * w);
+    for (int w = 0; w < P / 4; w++) qw[w] = ldg32(of.f1L + (size_t)q * P + 4 * w);
     const int px = gx << L, py = gy << L;
-    flow[q] = f;
-    cost[q] = sad_full<C>(f2L, make_tap<P>(px, py, flow_x(f), flow_y(f), L, WL, HL), qw);
+    of.flow[q] = f;
+    of.cost[q] = sad_full<C>(of.f2L, make_tap<P>(px, py, flow_x(f), flow_y(f), L, WL, HL), qw);
 }
 
 #include "ff_sweep.cuh"
@@ -455,13 +463,22 @@ __global__ void k_sparsify(const uint32_t *__restrict__ fwd, const uint32_t *__r
         for (int x = cx; x < x1; x++) mask_out[y * W + x] = (y * W + x == best) ? 1 : 0;
 }
 
-// level state -> caller's flow / cost arrays
-__global__ void k_export(const uint32_t *__restrict__ flow, const int *__restrict__ cost, int N,
-                         uint32_t *__restrict__ flow_out, int *__restrict__ cost_out) {
+// level state -> caller's flow / cost arrays; blockIdx.y: which of the flows
+struct ExportDir {
+    const uint32_t *flow;
+    const int *cost;
+    uint32_t *flow_out;
+    int *cost_out;
+};
+struct ExportArgs {
+    ExportDir of[3];
+};
+__global__ void k_export(const __grid_constant__ ExportArgs a, int N) {
+    const ExportDir &of = a.of[blockIdx.y];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    flow_out[i] = flow[i];
-    if (cost_out) cost_out[i] = cost[i];
+    of.flow_out[i] = of.flow[i];
+    if (of.cost_out) of.cost_out[i] = of.cost[i];
 }
 
 // Sec. 3.7 forward/backward consistency: keep p iff |F(p) + F_b(q)|^2 < eps^2
@@ -928,19 +945,27 @@ ff_status launch_search(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L
     return check_launch(c, "k_search");
 }
 
-ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L, uint32_t *flow,
-                       int *cost, int W, int H, int L, int t, uint32_t pair_id) {
-    DirState &st = c->dir[d];
+// A level's state of one of the flows in work.
+struct LevelDir {
+    int d;
+    const uint8_t *f1L, *f2L;
+    uint32_t *flow;
+    int *cost;
+};
+
+// One sweep of `nd` flows of a pair in the layout for many pairs in flight.
+ff_status launch_sweep_many(ff_ctx *c, const LevelDir *dirs, int nd, int W, int H, int L, int t,
+                            uint32_t pair_id) {
     int WL, HL;
     level_dims(W, H, L, &WL, &HL);
     SweepArgs a;
-    a.f1L = f1L;
-    a.f2L = f2L;
-    a.flow = flow;
-    a.cost = cost;
-    a.edge = st.edge;
-    a.ticket = st.ticket + (size_t)L * kMaxIters + t;
-    a.err = st.err;
+    a.dirs = nd;
+    for (int k = 0; k < nd; k++) {
+        DirState &st = c->dir[dirs[k].d];
+        a.of[k] = {dirs[k].f1L, dirs[k].f2L, dirs[k].flow, dirs[k].cost, st.edge,
+                   st.ticket + (size_t)L * kMaxIters + t, st.err, dirs[k].d};
+    }
+    for (int k = nd; k < kSweepDirs; k++) a.of[k] = a.of[0];
     a.W = W;
     a.H = H;
     a.L = L;
@@ -948,7 +973,6 @@ ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L,
     a.HL = HL;
     a.d = t & 3;
     a.t = t;
-    a.dir = d;
     a.do_rs = search_after(c->cfg, L, t) ? 1 : 0;
     a.radius_q3 = search_radius(c->cfg, L, t);
     a.seed = c->cfg.seed;
@@ -962,9 +986,9 @@ ff_status launch_sweep(ff_ctx *c, int d, const uint8_t *f1L, const uint8_t *f2L,
     const int nstrips = (HL + SweepGeo<1>::RW - 1) / SweepGeo<1>::RW;
     prof_begin(c, "k_sweep");
     if (c->C == 1)
-        k_sweep_many<1><<<nstrips, SweepGeo<1>::THREADS, 0, c->stream>>>(a);
+        k_sweep_many<1><<<nstrips * nd, SweepGeo<1>::THREADS, 0, c->stream>>>(a);
     else
-        k_sweep_many<3><<<nstrips, SweepGeo<3>::THREADS, 0, c->stream>>>(a);
+        k_sweep_many<3><<<nstrips * nd, SweepGeo<3>::THREADS, 0, c->stream>>>(a);
     return check_launch(c, "k_sweep");
 }
 
@@ -977,14 +1001,20 @@ void launch_given(ff_ctx *c, const uint32_t *seeds, const uint8_t *f1L, const ui
                                                           cost);
 }
 
-template <int C>
-void launch_upsample(ff_ctx *c, const uint32_t *pflow, int WP, const uint8_t *f1L,
-                     const uint8_t *f2L, int W, int H, int L, int WL, int HL, uint32_t *flow,
-                     int *cost) {
-    const int nq = WL * HL;
+ff_status launch_upsample(ff_ctx *c, const LevelDir *dirs, const uint32_t *const *pflow, int nd,
+                          int WP, int W, int H, int L, int WL, int HL) {
+    UpsampleArgs a;
+    for (int k = 0; k < 3; k++) {
+        const int j = k < nd ? k : 0;
+        a.of[k] = {pflow[j], dirs[j].f1L, dirs[j].f2L, dirs[j].flow, dirs[j].cost};
+    }
+    const dim3 grid((WL * HL + 255) / 256, nd);
     prof_begin(c, "k_upsample");
-    k_upsample<C><<<(nq + 255) / 256, 256, 0, c->stream>>>(pflow, WP, f1L, f2L, W, H, L, WL, HL,
-                                                        flow, cost);
+    if (c->C == 1)
+        k_upsample<1><<<grid, 256, 0, c->stream>>>(a, WP, W, H, L, WL, HL);
+    else
+        k_upsample<3><<<grid, 256, 0, c->stream>>>(a, WP, W, H, L, WL, HL);
+    return check_launch(c, "k_upsample");
 }
 
 ff_status check_pair(ff_ctx *c) {
@@ -995,78 +1025,106 @@ ff_status check_pair(ff_ctx *c) {
     return FF_OK;
 }
 
-ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seeds_in,
-                    int until_level, int until_sweeps, int16_t *flow_out, int32_t *cost_out) {
+// What one flow of a match starts from and where it goes.
+struct MatchDir {
+    ff_dir dir;
+    const int16_t *seeds_in;
+    int16_t *flow_out;
+    int32_t *cost_out;
+};
+
+// `nd` flows of a pair up to the given level and sweep, on the context's stream.
+// In the layout for many pairs in flight every level runs them in the same
+// launches; otherwise there is one.
+ff_status run_match_dirs(ff_ctx *c, const MatchDir *m, int nd, uint32_t pair_id, int until_level,
+                         int until_sweeps) {
     ff_status s = check_pair(c);
     if (s) return s;
-    if (dir != FF_FWD && dir != FF_BWD && dir != FF_BWD2)
-        return fail(c, FF_EINVAL, "dir must be FF_FWD, FF_BWD or FF_BWD2");
-    if (until_level < final_level(c->cfg) || until_level >= c->S || until_sweeps < 0 ||
-        until_sweeps > level_sweeps(c->cfg, until_level))
-        return fail(c, FF_EINVAL, "until_level/until_sweeps out of range");
-    if (!flow_out) return fail(c, FF_EINVAL, "flow_out is NULL");
-    if (((uintptr_t)flow_out & 3) || ((uintptr_t)cost_out & 3) || ((uintptr_t)seeds_in & 3))
-        return fail(c, FF_EINVAL, "flow_out, cost_out and seeds_in must be 4-byte aligned");
-    const int d = (int)dir;
+    for (int k = 0; k < nd; k++) {
+        if (m[k].dir != FF_FWD && m[k].dir != FF_BWD && m[k].dir != FF_BWD2)
+            return fail(c, FF_EINVAL, "dir must be FF_FWD, FF_BWD or FF_BWD2");
+        if (until_level < final_level(c->cfg) || until_level >= c->S || until_sweeps < 0 ||
+            until_sweeps > level_sweeps(c->cfg, until_level))
+            return fail(c, FF_EINVAL, "until_level/until_sweeps out of range");
+        if (!m[k].flow_out) return fail(c, FF_EINVAL, "flow_out is NULL");
+        if (((uintptr_t)m[k].flow_out & 3) || ((uintptr_t)m[k].cost_out & 3) ||
+            ((uintptr_t)m[k].seeds_in & 3))
+            return fail(c, FF_EINVAL, "flow_out, cost_out and seeds_in must be 4-byte aligned");
+    }
+    const bool block = c->sweep_lanes != 2;
     const int W = c->fw[0], H = c->fh[0];
-    const uint8_t *fsrc = c->feat[d == 0 ? 0 : 1];
-    const uint8_t *fdst = c->feat[d == 0 ? 1 : 0];
-    DirState &st = c->dir[d];
-    s = check_cuda(c, cudaMemsetAsync(st.ticket, 0, sizeof(unsigned) * FF_MAX_SCALES * kMaxIters,
-                                      c->stream),
-                   "memset tickets");
-    if (s) return s;
-    s = check_cuda(c, cudaMemsetAsync(st.edge, 0, c->edge_cap * sizeof(unsigned long long),
-                                      c->stream),
-                   "clear boundary rows");
-    if (s) return s;
+    for (int k = 0; k < nd; k++) {
+        DirState &st = c->dir[m[k].dir];
+        s = check_cuda(c, cudaMemsetAsync(st.ticket, 0,
+                                          sizeof(unsigned) * FF_MAX_SCALES * kMaxIters, c->stream),
+                       "memset tickets");
+        if (s) return s;
+        s = check_cuda(c, cudaMemsetAsync(st.edge, 0, c->edge_cap * sizeof(unsigned long long),
+                                          c->stream),
+                       "clear boundary rows");
+        if (s) return s;
+    }
     int cur = 0, WP = 0;
     for (int L = c->S - 1; L >= until_level; L--) {
         int WL, HL;
         level_dims(W, H, L, &WL, &HL);
         const size_t off = level_offset(W, H, c->P, L);
-        const uint8_t *f1L = fsrc + off, *f2L = fdst + off;
-        uint32_t *flow = st.flow[cur];
-        int *cost = st.cost[cur];
-        if (L == c->S - 1) {
-            if (seeds_in) {
-                if (c->C == 1)
-                    launch_given<1>(c, (const uint32_t *)seeds_in, f1L, f2L, W, H, L, WL, HL, flow,
-                                    cost);
-                else
-                    launch_given<3>(c, (const uint32_t *)seeds_in, f1L, f2L, W, H, L, WL, HL, flow,
-                                    cost);
-                s = check_launch(c, "k_seed_given");
-            } else {
-                const KnnOut out{c->cfg.seed_leaf, nullptr, nullptr, f1L, f2L, W, H, L,
-                                 WL, HL, flow, cost};
-                s = c->C == 1 ? launch_seed<1>(c, d, fsrc, fdst, W, H, out)
-                              : launch_seed<3>(c, d, fsrc, fdst, W, H, out);
-            }
-        } else {
-            if (c->C == 1)
-                launch_upsample<1>(c, st.flow[cur ^ 1], WP, f1L, f2L, W, H, L, WL, HL, flow, cost);
-            else
-                launch_upsample<3>(c, st.flow[cur ^ 1], WP, f1L, f2L, W, H, L, WL, HL, flow, cost);
-            s = check_launch(c, "k_upsample");
+        LevelDir dirs[kNumDirs];
+        const uint32_t *pflow[kNumDirs];
+        for (int k = 0; k < nd; k++) {
+            const int d = (int)m[k].dir;
+            DirState &st = c->dir[d];
+            dirs[k] = {d, c->feat[d == 0 ? 0 : 1] + off, c->feat[d == 0 ? 1 : 0] + off,
+                       st.flow[cur], st.cost[cur]};
+            pflow[k] = st.flow[cur ^ 1];
         }
-        if (s) return s;
+        if (L == c->S - 1) {
+            for (int k = 0; k < nd; k++) {
+                const LevelDir &v = dirs[k];
+                if (m[k].seeds_in) {
+                    if (c->C == 1)
+                        launch_given<1>(c, (const uint32_t *)m[k].seeds_in, v.f1L, v.f2L, W, H, L,
+                                        WL, HL, v.flow, v.cost);
+                    else
+                        launch_given<3>(c, (const uint32_t *)m[k].seeds_in, v.f1L, v.f2L, W, H, L,
+                                        WL, HL, v.flow, v.cost);
+                    s = check_launch(c, "k_seed_given");
+                } else {
+                    const KnnOut out{c->cfg.seed_leaf, nullptr, nullptr, v.f1L, v.f2L, W, H, L,
+                                     WL, HL, v.flow, v.cost};
+                    const uint8_t *fs = c->feat[v.d == 0 ? 0 : 1], *fd = c->feat[v.d == 0 ? 1 : 0];
+                    s = c->C == 1 ? launch_seed<1>(c, v.d, fs, fd, W, H, out)
+                                  : launch_seed<3>(c, v.d, fs, fd, W, H, out);
+                }
+                if (s) return s;
+            }
+        } else if ((s = launch_upsample(c, dirs, pflow, nd, WP, W, H, L, WL, HL))) {
+            return s;
+        }
         const int sweeps = (L == until_level) ? until_sweeps : level_sweeps(c->cfg, L);
-        const bool block = c->sweep_lanes != 2;
         for (int t = 0; t < sweeps; t++) {
-            if (!block)
-                s = launch_sweep(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
-            else if (c->C == 1)
-                s = launch_sweep_block<1>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
-            else
-                s = launch_sweep_block<3>(c, d, f1L, f2L, flow, cost, W, H, L, t, pair_id);
-            if (s) return s;
+            if (!block) {
+                if ((s = launch_sweep_many(c, dirs, nd, W, H, L, t, pair_id))) return s;
+                continue;
+            }
+            for (int k = 0; k < nd; k++) {
+                const LevelDir &v = dirs[k];
+                s = c->C == 1 ? launch_sweep_block<1>(c, v.d, v.f1L, v.f2L, v.flow, v.cost, W, H, L,
+                                                      t, pair_id)
+                              : launch_sweep_block<3>(c, v.d, v.f1L, v.f2L, v.flow, v.cost, W, H, L,
+                                                      t, pair_id);
+                if (s) return s;
+            }
         }
         if (block && sweeps > 0 && search_after(c->cfg, L, sweeps - 1)) {
-            s = c->C == 1
-                    ? launch_search<1>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id)
-                    : launch_search<3>(c, d, f1L, f2L, flow, cost, W, H, L, sweeps - 1, pair_id);
-            if (s) return s;
+            for (int k = 0; k < nd; k++) {
+                const LevelDir &v = dirs[k];
+                s = c->C == 1 ? launch_search<1>(c, v.d, v.f1L, v.f2L, v.flow, v.cost, W, H, L,
+                                                 sweeps - 1, pair_id)
+                              : launch_search<3>(c, v.d, v.f1L, v.f2L, v.flow, v.cost, W, H, L,
+                                                 sweeps - 1, pair_id);
+                if (s) return s;
+            }
         }
         WP = WL;
         if (L > until_level) cur ^= 1;
@@ -1074,10 +1132,21 @@ ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seed
     int WL, HL;
     level_dims(W, H, until_level, &WL, &HL);
     const int N = WL * HL;
+    ExportArgs x;
+    for (int k = 0; k < 3; k++) {
+        const MatchDir &o = m[k < nd ? k : 0];
+        DirState &st = c->dir[o.dir];
+        x.of[k] = {st.flow[cur], st.cost[cur], (uint32_t *)o.flow_out, (int *)o.cost_out};
+    }
     prof_begin(c, "k_export");
-    k_export<<<(N + 255) / 256, 256, 0, c->stream>>>(st.flow[cur], st.cost[cur], N,
-                                                     (uint32_t *)flow_out, (int *)cost_out);
+    k_export<<<dim3((N + 255) / 256, nd), 256, 0, c->stream>>>(x, N);
     return check_launch(c, "k_export");
+}
+
+ff_status run_match(ff_ctx *c, ff_dir dir, uint32_t pair_id, const int16_t *seeds_in,
+                    int until_level, int until_sweeps, int16_t *flow_out, int32_t *cost_out) {
+    const MatchDir m{dir, seeds_in, flow_out, cost_out};
+    return run_match_dirs(c, &m, 1, pair_id, until_level, until_sweeps);
 }
 
 ff_status filter_into(ff_ctx *c, const int16_t *fwd, const int16_t *b1, const int16_t *b2,
@@ -1087,7 +1156,8 @@ ff_status region_into(ff_ctx *c, const int16_t *fwd, const uint8_t *mask_in, int
 
 // One whole pair on device buffers, enqueued without waiting: features on
 // the context's stream, the backward flow(s) on the side stream(s)
-// overlapping the forward flow, the filter after all of them.  The next
+// overlapping the forward flow (in a slot: every flow on the one stream, in the
+// same launches), the filter after all of them.  The next
 // work on the context's stream is ordered after every part.
 ff_status enqueue_pair(ff_ctx *c, const uint8_t *img1, const uint8_t *img2, int w, int h,
                        int pitch, uint32_t pair_id, int16_t *fwd, int16_t *bwd, int16_t *bwd2,
@@ -1096,6 +1166,19 @@ ff_status enqueue_pair(ff_ctx *c, const uint8_t *img1, const uint8_t *img2, int 
     const int n = level_sweeps(c->cfg, Lf);
     cudaStream_t main = c->stream;
     ff_status s;
+    if (c->sweep_lanes == 2) {
+        // many pairs in flight: one stream per pair, its flows in the same launches
+        if ((s = ff_features(c, 0, img1, w, h, pitch))) return s;
+        if ((s = ff_features(c, 1, img2, w, h, pitch))) return s;
+        const MatchDir m[kNumDirs] = {{FF_FWD, nullptr, fwd, nullptr},
+                                      {FF_BWD, nullptr, bwd, nullptr},
+                                      {FF_BWD2, nullptr, bwd2, nullptr}};
+        if ((s = run_match_dirs(c, m, bwd2 ? 3 : 2, pair_id, Lf, n))) return s;
+        if (!mask) return FF_OK;
+        if ((s = filter_into(c, fwd, bwd, bwd2, mask))) return s;
+        if (c->cfg.region_min > 0) return region_into(c, fwd, mask, c->cfg.region_min, mask);
+        return FF_OK;
+    }
     // the two frames' features on the two streams (the side stream starts
     // after what main holds so far), then each stream waits for the other's
     if ((s = check_cuda(c, cudaEventRecord(c->ev_a, main), "event"))) return s;

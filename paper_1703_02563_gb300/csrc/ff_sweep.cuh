@@ -5,7 +5,12 @@
 
 namespace ffk {
 
-struct SweepArgs {
+// One launch runs the same sweep of up to kSweepDirs flows of a pair (its CTAs
+// alternate between them): the flows then need one stream and one launch, where a
+// stream each (three per slot) shared the few hardware queues a process has by
+// default, and pairs in flight waited for one another.
+constexpr int kSweepDirs = 3;
+struct SweepDir {
     const uint8_t *f1L;
     const uint8_t *f2L;
     uint32_t *flow;                // level state, updated in place
@@ -13,8 +18,13 @@ struct SweepArgs {
     unsigned long long *edge;      // [nstrips][WL] boundary rows: (epoch << 32) | flow
     unsigned int *ticket;          // strip counter of this launch (zeroed before)
     int *err;                      // error word of this direction
+    int dir;
+};
+struct SweepArgs {
+    SweepDir of[kSweepDirs];
+    int dirs;
     int W, H, L, WL, HL;
-    int d, t, dir, do_rs, radius_q3;
+    int d, t, do_rs, radius_q3;
     uint32_t seed, pair_id, epoch;
     unsigned long long wait_ns;
     int force_timeout;
@@ -234,7 +244,7 @@ __device__ __forceinline__ bool wait_expired(unsigned long long &t0, unsigned lo
 // Bounded to the registers that let MIN_CTAS CTAs share an SM.
 template <int C>
 __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
-    k_sweep_many(const SweepArgs a) {
+    k_sweep_many(const __grid_constant__ SweepArgs a) {
     using SG = SweepGeo<C>;
     constexpr int P = SG::P, G = SG::G, RW = SG::RW;
     constexpr int DI = SG::DI, DO = SG::DO, A = SG::A, LRING = SG::LRING;
@@ -246,11 +256,12 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
     volatile int *v_lcons = &sm.lcons;
     volatile int *v_abort = &sm.abort;
 
+    const SweepDir &of = a.of[blockIdx.x % (unsigned)a.dirs];
     const int tid = threadIdx.x;
     const int U = a.WL, V = a.HL;
     const int nstrips = (V + RW - 1) / RW;
     if (tid == 0) {
-        sm.strip = (int)atomicAdd(a.ticket, 1u);
+        sm.strip = (int)atomicAdd(of.ticket, 1u);
         sm.lcons = 0;
         sm.abort = 0;
         sm.in_ready = 0;
@@ -268,7 +279,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
     if (warp == SG::LOADER) {
         // ---------------- loader warp: previous strip's last row -> lring
         if (strip == 0) return;
-        const unsigned long long *src = a.edge + (size_t)(strip - 1) * U;
+        const unsigned long long *src = of.edge + (size_t)(strip - 1) * U;
         const uint32_t want = (a.force_timeout && strip == 1) ? (a.epoch ^ 0x80000000u) : a.epoch;
         int base = 0;
         unsigned long long t0 = globaltimer_ns();
@@ -294,8 +305,8 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                 int stop = 0;
                 if (lane == 0) {
                     const bool late = globaltimer_ns() - t0 > a.wait_ns;
-                    if (late) atomicCAS(a.err, 0, kErrTimeout);
-                    stop = late || *v_abort || ld_relaxed_i32(a.err) != 0;
+                    if (late) atomicCAS(of.err, 0, kErrTimeout);
+                    stop = late || *v_abort || ld_relaxed_i32(of.err) != 0;
                     if (stop) *v_abort = 1;
                 }
                 if (__shfl_sync(FULL, stop, 0)) return;
@@ -314,7 +325,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
     const int gy = row_ok ? (flipy ? V - 1 - v : v) : 0;
     const int py = gy * n;
     const int NS = U + RW - 1;                            // local steps of a warp
-    const uint8_t *f1L = a.f1L, *f2L = a.f2L;
+    const uint8_t *f1L = of.f1L, *f2L = of.f2L;
     const size_t rowbase = (size_t)gy * U;
 
     if (warp == 2) {
@@ -329,8 +340,8 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                 const int gx = flipx ? U - 1 - uj : uj;
                 const size_t pi = rowbase + gx;
                 const int slot = j & (DI - 1);
-                if (g == 0) cp_async4(&sm.in_flow[slot][k], a.flow + pi);
-                if (g == G - 1) cp_async4(&sm.in_cost[slot][k], a.cost + pi);
+                if (g == 0) cp_async4(&sm.in_flow[slot][k], of.flow + pi);
+                if (g == G - 1) cp_async4(&sm.in_cost[slot][k], of.cost + pi);
                 uint8_t *dst = &sm.in_raw[slot][k][QB * g];
                 const uint8_t *srcq = f1L + pi * P + QB * g;
                 if constexpr (QB == 16) cp_async16ca(dst, srcq);
@@ -360,7 +371,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                 while (true) {
                     ocons = *v_out_cons;
                     if (__all_sync(FULL, ocons > j - DI)) break;
-                    if (wait_expired(t0, a.wait_ns, v_abort, a.err)) {
+                    if (wait_expired(t0, a.wait_ns, v_abort, of.err)) {
                         cp_async_wait<0>();
                         return;
                     }
@@ -395,7 +406,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                     const int gxp = flipx ? U - 1 - up : up;
                     const uint4 rnd = philox4x32_10(
                         make_uint4((uint32_t)(py * W + gxp * n), (uint32_t)a.t, (uint32_t)L,
-                                   (uint32_t)a.dir),
+                                   (uint32_t)of.dir),
                         a.seed, a.pair_id);
                     const int ox = (int)(rnd.x % span) - Rq, oy = (int)(rnd.y % span) - Rq;
                     offs[j] = (ox & 0xffff) | (oy << 16);
@@ -409,7 +420,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                 e = lds64(oslot);
                 const bool ok = (uint32_t)(e >> 52) == (uint32_t)(i & 0xFFF);
                 if (__all_sync(FULL, ok)) break;
-                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+                if (wait_expired(t0, a.wait_ns, v_abort, of.err)) return;
             }
             int4 nq[WPH];
 #pragma unroll
@@ -451,8 +462,8 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
                 }
             }
             if (valid && g == 0) {
-                a.flow[rowbase + gx] = fflow;
-                a.cost[rowbase + gx] = fcost;
+                of.flow[rowbase + gx] = fflow;
+                of.cost[rowbase + gx] = fcost;
             }
         }
         return;
@@ -488,7 +499,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
         if (!__all_sync(FULL, ok)) {
             unsigned long long t0 = 0;
             while (true) {
-                if (wait_expired(t0, a.wait_ns, v_abort, a.err)) return;
+                if (wait_expired(t0, a.wait_ns, v_abort, of.err)) return;
                 ready = *v_in_ready;
                 ocons = *v_out_cons;
                 ok = ready > i && ocons > i - DO;
@@ -534,7 +545,7 @@ __global__ void __launch_bounds__(SweepGeo<C>::THREADS, SweepGeo<C>::MIN_CTAS)
         }
         if (active) last = best;
         // the strip's last row -> the next strip (a predicated store)
-        st_relaxed_u64_if(a.edge + (size_t)strip * U + uc, ((unsigned long long)a.epoch << 32) | best,
+        st_relaxed_u64_if(of.edge + (size_t)strip * U + uc, ((unsigned long long)a.epoch << 32) | best,
                           edge_out && active && g == 0);
         // result -> random-search warp (tagged slot)
         if (g == 0) sts64(&sm.out[i & (DO - 1)][k], pack_out(i, bcost, best));
