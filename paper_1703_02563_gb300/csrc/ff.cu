@@ -122,99 +122,95 @@ __global__ void k_dense(const uint8_t *__restrict__ feat, int N, int8_t *__restr
 // Sec. 3.2 Eq. 4; kd-tree leaf replaced by the exact nearest neighbours it
 // approximates); the contexts' own search is in ff_seed_tc.cuh
 // ---------------------------------------------------------------------------
-// insert (d, i) into the ascending list (D, I) of 8, dropping the last entry
-__device__ __forceinline__ void list_insert(int (&D)[8], int (&I)[8], int d, int i) {
-#pragma unroll
-    for (int k = 0; k < 8; k++) {
-        const bool sw = lex_less(d, i, D[k], I[k]);
-        const int td = D[k], ti = I[k];
-        D[k] = sw ? d : td;
-        I[k] = sw ? i : ti;
-        d = sw ? td : d;
-        i = sw ? ti : i;
-    }
-}
-
-// Phase 1: QPT queries per thread (a tile of 128*QPT queries per CTA), one
-// candidate chunk per blockIdx.y.  Candidates of the chunk are staged 256 at
-// a time in shared memory with their squared norms.  Since
-// |q - c|^2 = |q|^2 + |c|^2 - 2 q.c and |q|^2 is fixed per query, the lists
-// are kept on the key |c|^2 - 2 q.c (one dp4a per 4 dimensions for q.c) and
-// |q|^2 is added on output.  Within a chunk candidates arrive in increasing
-// linear index, so a strict compare against the list's worst key keeps the
-// (distance, index) order.
+// As the tensor-core form keeps, per query, the tiles of consecutive candidates
+// with the least (least key, tile) -- key = |c|^2 - 2 q.c, one dp4a per 4
+// dimensions -- for k_seed_pick to rank (ff_seed_tc.cuh has the argument), but
+// without tiles of its own in memory: QPT queries per thread, one chunk of tiles per
+// blockIdx.y, 128 candidates at a time staged in shared memory with their norms in
+// the row's free last word.  A tile has `trows` candidates, a multiple of 128.
+//
+// What bounds it: the dp4a and minimum per candidate and query (exact lists of
+// candidates, kept here before, took their insertion path for most candidates
+// of a warp: 605 us at 640x480 gray, every second candidate).
 template <int C, int QPT>
 __global__ void __launch_bounds__(128)
     k_seed_scan(const uint8_t *__restrict__ f1, const uint8_t *__restrict__ f2, int W, int N,
-                int WS, int NQ, int stride, int Wc, int ncand, int chunk, int2 *__restrict__ part) {
-    constexpr int P = Geo<C>::P, NV = P / 16, NW = Geo<C>::NW, TILE = 256;
-    __shared__ uint4 s_w[TILE][NV];
-    __shared__ int2 s_ni[TILE];   // (norm, linear index)
-    uint32_t qw[QPT][NW];
-    int thr[QPT];
-    int D[QPT][8], I[QPT][8];
+                int WS, int NQ, int stride, int Wc, int ncand, int trows, int chunk,
+                uint32_t *__restrict__ lists, int nqpad) {
+    constexpr int P = Geo<C>::P, NV = P / 16, NW = Geo<C>::NW;
+    constexpr int kMissing = 0x3fffffff;   // norm of a row past the end
+    __shared__ uint4 s_w[kTcRows][NV];
+    uint32_t qw[QPT][NW], l[QPT][8];
+    int least[QPT];
 #pragma unroll
     for (int j = 0; j < QPT; j++) {
         const int q = min((blockIdx.x * QPT + j) * 128 + threadIdx.x, NQ - 1);
         const int gy = q / WS, gx = q - gy * WS;
         const uint32_t *src =
-            reinterpret_cast<const uint32_t *>(f1 + ((size_t)gy * N * W + gx * N) * P);
-        int qn = 0;
+            reinterpret_cast<const uint32_t *>(f1 + ((size_t)gy * N * W + (size_t)gx * N) * P);
 #pragma unroll
-        for (int w = 0; w < NW; w++) {
-            qw[j][w] = __ldg(src + w);
-            qn = __dp4a((int)qw[j][w], (int)qw[j][w], qn);
-        }
-        (void)qn;
-        thr[j] = 0x7fffffff;   // the list's worst key; INT32_MAX while not full
+        for (int w = 0; w < NW; w++) qw[j][w] = __ldg(src + w);
 #pragma unroll
-        for (int k = 0; k < 8; k++) D[j][k] = I[j][k] = 0x7fffffff;
+        for (int e = 0; e < 8; e++) l[j][e] = 0xffffffffu;
+        least[j] = kMissing;
     }
-    const int c0 = blockIdx.y * chunk, c1 = min(c0 + chunk, ncand);
-    for (int base = c0; base < c1; base += TILE) {
+    const int tile0 = blockIdx.y * chunk;
+    const int c0 = tile0 * trows, c1 = min(c0 + chunk * trows, ncand);
+    for (int base = c0; base < c1; base += kTcRows) {
         __syncthreads();
-        for (int k = threadIdx.x; k < TILE; k += 128) {
-            const int ci = base + k;
+        {
+            const int ci = base + threadIdx.x;
+            uint4 r[NV];
+#pragma unroll
+            for (int v = 0; v < NV; v++) r[v] = make_uint4(0, 0, 0, 0);
+            int nn = kMissing;
             if (ci < c1) {
-                const int cy = (ci / Wc) * stride, cx = (ci % Wc) * stride;
-                const uint4 *src = reinterpret_cast<const uint4 *>(f2 + ((size_t)cy * W + cx) * P);
-                int nn = 0;
+                const int cy = ci / Wc, cx = ci - cy * Wc;
+                const uint4 *src = reinterpret_cast<const uint4 *>(
+                    f2 + ((size_t)cy * stride * W + (size_t)cx * stride) * P);
+                nn = 0;
 #pragma unroll
                 for (int v = 0; v < NV; v++) {
-                    const uint4 x = __ldg(src + v);
-                    s_w[k][v] = x;
-                    nn = __dp4a((int)x.x, (int)x.x, nn);
-                    nn = __dp4a((int)x.y, (int)x.y, nn);
-                    nn = __dp4a((int)x.z, (int)x.z, nn);
-                    nn = __dp4a((int)x.w, (int)x.w, nn);
+                    r[v] = __ldg(src + v);
+                    nn = __dp4a((int)r[v].x, (int)r[v].x, nn);
+                    nn = __dp4a((int)r[v].y, (int)r[v].y, nn);
+                    nn = __dp4a((int)r[v].z, (int)r[v].z, nn);
+                    nn = __dp4a((int)r[v].w, (int)r[v].w, nn);
                 }
-                s_ni[k] = make_int2(nn, cy * W + cx);
             }
+            r[NV - 1].w = (uint32_t)nn;
+#pragma unroll
+            for (int v = 0; v < NV; v++) s_w[threadIdx.x][v] = r[v];
         }
         __syncthreads();
-        const int cnt = min(TILE, c1 - base);
-        for (int k = 0; k < cnt; k++) {
+#pragma unroll 4
+        for (int k = 0; k < kTcRows; k++) {
             uint32_t cw[NV * 4];
 #pragma unroll
             for (int v = 0; v < NV; v++) {
                 const uint4 x = s_w[k][v];
-                cw[4 * v] = x.x;
-                cw[4 * v + 1] = x.y;
-                cw[4 * v + 2] = x.z;
-                cw[4 * v + 3] = x.w;
+                cw[4 * v] = x.x, cw[4 * v + 1] = x.y, cw[4 * v + 2] = x.z, cw[4 * v + 3] = x.w;
             }
-            const int2 ni = s_ni[k];
 #pragma unroll
             for (int j = 0; j < QPT; j++) {
                 int dot = 0;
 #pragma unroll
                 for (int w = 0; w < NW; w++) dot = __dp4a((int)qw[j][w], (int)cw[w], dot);
-                const int key = ni.x - 2 * dot;
-                if (key < thr[j]) {
-                    // the list stores |c|^2 - 2 q.c; |q|^2 is added on output
-                    list_insert(D[j], I[j], key, ni.y);
-                    thr[j] = D[j][7];
+                least[j] = min(least[j], (int)cw[NV * 4 - 1] - 2 * dot);
+            }
+        }
+        if ((base + kTcRows - c0) % trows == 0 || base + kTcRows >= c1) {   // a tile ends
+            const uint32_t t = (uint32_t)((base - c0) / trows);
+#pragma unroll
+            for (int j = 0; j < QPT; j++) {
+                uint32_t x = ((uint32_t)(least[j] + kTcKeyBias) << kTcTileBits) + t;
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    const uint32_t lo = min(l[j][e], x);
+                    x = max(l[j][e], x);
+                    l[j][e] = lo;
                 }
+                least[j] = kMissing;
             }
         }
     }
@@ -222,37 +218,9 @@ __global__ void __launch_bounds__(128)
     for (int j = 0; j < QPT; j++) {
         const int q = (blockIdx.x * QPT + j) * 128 + threadIdx.x;
         if (q >= NQ) continue;
-        int qn = 0;
-#pragma unroll
-        for (int w = 0; w < NW; w++) qn = __dp4a((int)qw[j][w], (int)qw[j][w], qn);
-        int2 *dst = part + ((size_t)blockIdx.y * NQ + q) * 8;
-#pragma unroll
-        for (int k = 0; k < 8; k++)
-            dst[k] = make_int2(I[j][k] == 0x7fffffff ? 0x7fffffff : D[j][k] + qn, I[j][k]);
-    }
-}
-
-// Phase 2: merge the per-chunk lists of each query into its top-l.
-__global__ void k_seed_merge(const int2 *__restrict__ part, int nchunks, int NQ, int leaf,
-                             int *__restrict__ knn_idx, int *__restrict__ knn_dist) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= NQ) return;
-    int D[8], I[8];
-#pragma unroll
-    for (int k = 0; k < 8; k++) D[k] = I[k] = 0x7fffffff;
-    for (int c = 0; c < nchunks; c++) {
-        const int2 *src = part + ((size_t)c * NQ + q) * 8;
-        for (int k = 0; k < 8; k++) {
-            const int2 e = src[k];
-            if (e.y == 0x7fffffff) break;
-            if (!lex_less(e.x, e.y, D[7], I[7])) break;
-            list_insert(D, I, e.x, e.y);
-        }
-    }
-    for (int k = 0; k < leaf; k++) {
-        const bool ok = I[k] != 0x7fffffff;
-        knn_idx[(size_t)q * leaf + k] = ok ? I[k] : -1;
-        knn_dist[(size_t)q * leaf + k] = ok ? D[k] : -1;
+        uint4 *dst = reinterpret_cast<uint4 *>(lists + ((size_t)blockIdx.y * nqpad + q) * 8);
+        dst[0] = make_uint4(l[j][0], l[j][1], l[j][2], l[j][3]);
+        dst[1] = make_uint4(l[j][4], l[j][5], l[j][6], l[j][7]);
     }
 }
 
@@ -521,8 +489,7 @@ namespace {
 
 constexpr int kMaxIters = 64;
 constexpr int kNumDirs = 3;   // forward, backward, second backward
-constexpr int kMaxChunks = 64;
-constexpr int kCtasPerSm = 8;     // seeding grids: about this many CTAs per SM
+constexpr int kCtasPerSm = 4;     // grid of the allocation-free seeding: about this many CTAs per SM
 constexpr int kSeedQpt = 2;
 constexpr int kSeedQueriesPerCta = 128 * kSeedQpt;
 
@@ -780,18 +747,6 @@ ff_status validate_config(const ff_config *c, std::string *why) {
     return FF_OK;
 }
 
-// seeding launch geometry: queries in tiles of 128, candidates split so the
-// grid holds about kCtasPerSm CTAs per SM of the device (sms)
-void seed_geometry(int nq, int ncand, int sms, int *nchunks, int *chunk) {
-    const int qt = (nq + kSeedQueriesPerCta - 1) / kSeedQueriesPerCta;
-    int nc = (kCtasPerSm * sms + qt - 1) / qt;
-    nc = nc < 1 ? 1 : (nc > kMaxChunks ? kMaxChunks : nc);
-    int ch = (ncand + nc - 1) / nc;
-    if (ch < 512) ch = 512;
-    *chunk = ch;
-    *nchunks = (ncand + ch - 1) / ch;
-}
-
 // How the seeding's product is split: nqt tiles of 128 queries by nch chunks of
 // `chunk` tiles of 128 candidates.  Two CTAs share an SM, so `slots` run at
 // once; among the chunk counts the one whose waves take the fewest tiles is
@@ -856,7 +811,7 @@ ff_status launch_seed(ff_ctx *c, int d, const uint8_t *fs, const uint8_t *fd, in
     if ((s = check_launch(c, "k_seed_scan"))) return s;
     prof_begin(c, "k_seed_merge");
     k_seed_pick<C><<<(nq + 3) / 4, 128, 0, c->stream>>>(fs, fd, W, N, WS, nq, stride, Wc, ncand,
-                                                        st.lists, z.nqt, z.nch, z.chunk, out);
+                                                        st.lists, z.nqt, z.nch, z.chunk, kTcRows, out);
     return check_launch(c, "k_seed_merge");
 }
 
@@ -1772,28 +1727,43 @@ ff_status ff_seed_knn_static(const int8_t *feat_src0, const int8_t *feat_dst0, i
     const int N = 1 << (scales - 1);
     const int Wc = (w + stride - 1) / stride, Hc = (h + stride - 1) / stride;
     const int ncand = Wc * Hc;
-    int nchunks, chunk, sms = 0;
+    int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return *msg = "device query failed", FF_ECUDA;
-    seed_geometry((int)nq, ncand, sms, &nchunks, &chunk);
-    const int cap = (int)(max_slots / nq);
-    if (nchunks > cap) {
-        chunk = (ncand + cap - 1) / cap;
-        nchunks = (ncand + chunk - 1) / chunk;
-    }
+    // chunks for about kCtasPerSm CTAs per SM, as far as their lists fit the scratch;
+    // tiles long enough that a chunk's have numbers of kTcTileBits
+    const int nqt = ((int)nq + kTcRows - 1) / kTcRows, nqpad = nqt * kTcRows;
+    const int qt = ((int)nq + kSeedQueriesPerCta - 1) / kSeedQueriesPerCta;
+    const int cap = (int)(kStaticScratchInt2 * 2 / 8 / (size_t)nqpad);   // >= 1: nq is limited
+    const int rows = (ncand + kTcRows - 1) / kTcRows;
+    const int want = max(1, min(min(kCtasPerSm * sms / qt, cap), rows));
+    int trows = kTcRows;
+    while ((long long)trows * want * kTcChunkTiles < ncand) trows *= 2;
+    const int tiles = (ncand + trows - 1) / trows;
+    const int chunk = (tiles + want - 1) / want, nch = (tiles + chunk - 1) / chunk;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     const uint8_t *fs = (const uint8_t *)feat_src0, *fd = (const uint8_t *)feat_dst0;
-    dim3 grid((unsigned)((nq + kSeedQueriesPerCta - 1) / kSeedQueriesPerCta), nchunks);
+    uint32_t *lists = (uint32_t *)scratch;
+    const dim3 grid((unsigned)qt, nch);
     if (channels == 1)
         k_seed_scan<1, kSeedQpt><<<grid, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc,
-                                                          ncand, chunk, scratch);
+                                                          ncand, trows, chunk, lists, nqpad);
     else
         k_seed_scan<3, kSeedQpt><<<grid, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc,
-                                                          ncand, chunk, scratch);
+                                                          ncand, trows, chunk, lists, nqpad);
     if (cudaGetLastError() != cudaSuccess) return *msg = "k_seed_scan launch failed", FF_ECUDA;
-    k_seed_merge<<<(unsigned)((nq + 127) / 128), 128, 0, stream>>>(scratch, nchunks, (int)nq, leaf,
-                                                                  idx_out, dist_out);
-    if (cudaGetLastError() != cudaSuccess) return *msg = "k_seed_merge launch failed", FF_ECUDA;
+    KnnOut out{};
+    out.leaf = leaf;
+    out.idx = idx_out;
+    out.dist = dist_out;
+    const unsigned nb = (unsigned)((nq + 3) / 4);
+    if (channels == 1)
+        k_seed_pick<1><<<nb, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand, lists,
+                                               nqt, nch, chunk, trows, out);
+    else
+        k_seed_pick<3><<<nb, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand, lists,
+                                               nqt, nch, chunk, trows, out);
+    if (cudaGetLastError() != cudaSuccess) return *msg = "k_seed_pick launch failed", FF_ECUDA;
     return FF_OK;
 }
 

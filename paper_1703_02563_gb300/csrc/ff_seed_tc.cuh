@@ -417,12 +417,13 @@ __device__ __forceinline__ void knn_finish(const KnnOut &o, int q, int lane, Knn
 // A query's tile lists -> its top 8 (and, for a match, its coarsest flow); one
 // warp per query.  The eight tiles of least (key, tile) come from its nch
 // lists; the eighth's least key bounds the eighth distance, so few of their
-// 1024 candidates are kept: those are collected and sorted once.
+// candidates (8 x 128 from the tensor cores) are kept: those are collected and
+// sorted once.  A tile has `trows` candidates, a multiple of 128.
 template <int C>
 __global__ void __launch_bounds__(128)
     k_seed_pick(const uint8_t *__restrict__ fq, const uint8_t *__restrict__ fc, int W, int N,
                 int WS, int nq, int stride, int Wc, int ncand, const uint32_t *__restrict__ lists,
-                int nqt, int nch, int chunk, const KnnOut out) {
+                int nqt, int nch, int chunk, int trows, const KnnOut out) {
     constexpr int P = Geo<C>::P, NV = P / 16, NW = Geo<C>::NW;
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ int2 s_buf[4][32];
@@ -468,43 +469,45 @@ __global__ void __launch_bounds__(128)
     for (int k = 0; k < 8; k++) {
         const int t = __shfl_sync(FULL, best.I, k);
         if (t == 0x7fffffff) break;
-        uint4 r[4][NV];
-        int idx[4];
+        for (int o0 = t * trows; o0 < min((t + 1) * trows, ncand); o0 += kTcRows) {
+            uint4 r[4][NV];
+            int idx[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            idx[j] = min(t * kTcRows + 32 * j + lane, ncand - 1);
-            if (stride > 1) {
-                const int cy = idx[j] / Wc, cx = idx[j] - cy * Wc;
-                idx[j] = cy * stride * W + cx * stride;
+            for (int j = 0; j < 4; j++) {
+                idx[j] = min(o0 + 32 * j + lane, ncand - 1);
+                if (stride > 1) {
+                    const int cy = idx[j] / Wc, cx = idx[j] - cy * Wc;
+                    idx[j] = cy * stride * W + cx * stride;
+                }
+#pragma unroll
+                for (int v = 0; v < NV; v++)
+                    r[j][v] = __ldg(reinterpret_cast<const uint4 *>(fc + (size_t)idx[j] * P) + v);
             }
 #pragma unroll
-            for (int v = 0; v < NV; v++)
-                r[j][v] = __ldg(reinterpret_cast<const uint4 *>(fc + (size_t)idx[j] * P) + v);
-        }
+            for (int j = 0; j < 4; j++) {
+                int dot = 0, nn = 0;
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
-            int dot = 0, nn = 0;
-#pragma unroll
-            for (int w = 0; w < NW; w++) {
-                const uint32_t cw = reinterpret_cast<const uint32_t *>(&r[j][0])[w];
-                dot = __dp4a((int)cw, (int)qw[w], dot);
-                nn = __dp4a((int)cw, (int)cw, nn);
-            }
-            const int d = nn + qn - 2 * dot;
-            const bool hit = t * kTcRows + 32 * j + lane < ncand && lex_less(d, idx[j], bD, bI);
-            const unsigned m = __ballot_sync(FULL, hit);
-            if (!m) continue;
-            if (held + __popc(m) > 32) {   // full: into the list, which lowers the bound
-                __syncwarp();
-                const int2 e = lane < held ? buf[lane] : make_int2(0x7fffffff, 0x7fffffff);
-                knn_take(l, e.x, e.y, lane, bD, bI);
-                knn_take(l, hit ? d : 0x7fffffff, idx[j], lane, bD, bI);
-                held = 0;
-                const int D = __shfl_sync(FULL, l.D, 7), I = __shfl_sync(FULL, l.I, 7);
-                if (lex_less(D, I, bD, bI)) bD = D, bI = I;
-            } else {
-                if (hit) buf[held + __popc(m & ((1u << lane) - 1))] = make_int2(d, idx[j]);
-                held += __popc(m);
+                for (int w = 0; w < NW; w++) {
+                    const uint32_t cw = reinterpret_cast<const uint32_t *>(&r[j][0])[w];
+                    dot = __dp4a((int)cw, (int)qw[w], dot);
+                    nn = __dp4a((int)cw, (int)cw, nn);
+                }
+                const int d = nn + qn - 2 * dot;
+                const bool hit = o0 + 32 * j + lane < ncand && lex_less(d, idx[j], bD, bI);
+                const unsigned m = __ballot_sync(FULL, hit);
+                if (!m) continue;
+                if (held + __popc(m) > 32) {   // full: into the list, which lowers the bound
+                    __syncwarp();
+                    const int2 e = lane < held ? buf[lane] : make_int2(0x7fffffff, 0x7fffffff);
+                    knn_take(l, e.x, e.y, lane, bD, bI);
+                    knn_take(l, hit ? d : 0x7fffffff, idx[j], lane, bD, bI);
+                    held = 0;
+                    const int D = __shfl_sync(FULL, l.D, 7), I = __shfl_sync(FULL, l.I, 7);
+                    if (lex_less(D, I, bD, bI)) bD = D, bI = I;
+                } else {
+                    if (hit) buf[held + __popc(m & ((1u << lane) - 1))] = make_int2(d, idx[j]);
+                    held += __popc(m);
+                }
             }
         }
     }
