@@ -333,34 +333,57 @@ __device__ void rf_unite(int *parent, int a, int b) {
     }
 }
 
-__global__ void k_rf_init(const uint8_t *__restrict__ mask, int N, int *parent, int *size,
-                          uint8_t *flag) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    parent[i] = mask[i] ? i : -1;
+// neighbouring kept points of one region
+__device__ __forceinline__ bool rf_joined(const uint32_t *__restrict__ flow,
+                                          const uint8_t *__restrict__ mask, int a, int b) {
+    return mask[a] && mask[b] && rf_close(flow[a], flow[b]);
+}
+
+// A point starts under the first point of its horizontal run within its warp's 32
+// points, so that most unions along rows are never made.
+__global__ void k_rf_init(const uint32_t *__restrict__ flow, const uint8_t *__restrict__ mask,
+                          int W, int N, int *parent, int *size, uint8_t *flag) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+    const bool in = i < N;
+    const bool left = in && lane > 0 && i % W > 0 && rf_joined(flow, mask, i, i - 1);
+    const unsigned runs = ~__ballot_sync(0xffffffffu, left) & ((2u << lane) - 1u);   // run starts
+    if (!in) return;
+    parent[i] = mask[i] ? i - (lane - (31 - __clz(runs))) : -1;
     size[i] = 0;
     flag[i] = 0;
 }
 
+// The unions that k_rf_init left: along rows between warps, and between rows,
+// where a run's points below the first one that joins the run beneath add nothing.
 __global__ void k_rf_union(const uint32_t *__restrict__ flow, const uint8_t *__restrict__ mask,
                            int W, int H, int *parent) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= W * H || !mask[i]) return;
     const int y = i / W, x = i - y * W;
-    const uint32_t f = flow[i];
-    if (x + 1 < W && mask[i + 1] && rf_close(f, flow[i + 1])) rf_unite(parent, i, i + 1);
-    if (y + 1 < H && mask[i + W] && rf_close(f, flow[i + W])) rf_unite(parent, i, i + W);
+    const bool left = x > 0 && rf_joined(flow, mask, i, i - 1);
+    if (left && (threadIdx.x & 31) == 0) rf_unite(parent, i, i - 1);
+    if (y + 1 < H && rf_joined(flow, mask, i, i + W) &&
+        !(left && rf_joined(flow, mask, i + W, i + W - 1) &&
+          rf_joined(flow, mask, i - 1, i - 1 + W)))
+        rf_unite(parent, i, i + W);
 }
 
-// region sizes, and whether a region touches a joinable removed point
+// region sizes (one addition per region and warp: a large region's count is one
+// word, and its points' single additions took most of this filter's time), and
+// whether a region touches a joinable removed point
 __global__ void k_rf_count(const uint32_t *__restrict__ flow, const uint8_t *__restrict__ mask,
                            int W, int H, int *parent, int *size, uint8_t *flag) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= W * H || !mask[i]) return;
+    const bool kept = i < W * H && mask[i];
+    int r = -1;
+    if (kept) {
+        r = rf_find_halve(parent, i);
+        atomicMin(parent + i, r);
+    }
+    const unsigned same = __match_any_sync(0xffffffffu, r);
+    if (!kept) return;
+    if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(size + r, __popc(same));
     const int y = i / W, x = i - y * W;
-    const int r = rf_find_halve(parent, i);
-    atomicMin(parent + i, r);
-    atomicAdd(size + r, 1);
     const uint32_t f = flow[i];
     const int nb[4] = {x + 1 < W ? i + 1 : -1, x > 0 ? i - 1 : -1, y + 1 < H ? i + W : -1,
                        y > 0 ? i - W : -1};
@@ -1216,7 +1239,7 @@ ff_status region_into(ff_ctx *c, const int16_t *fwd, const uint8_t *mask_in, int
     const uint32_t *f = (const uint32_t *)fwd;
     ff_status st;
     prof_begin(c, "k_region");
-    k_rf_init<<<nb, 256, 0, c->stream>>>(mask_in, N, c->rf_parent, c->rf_size, c->rf_flag);
+    k_rf_init<<<nb, 256, 0, c->stream>>>(f, mask_in, W, N, c->rf_parent, c->rf_size, c->rf_flag);
     if ((st = check_launch(c, "k_region"))) return st;
     prof_begin(c, "k_region");
     k_rf_union<<<nb, 256, 0, c->stream>>>(f, mask_in, W, H, c->rf_parent);
