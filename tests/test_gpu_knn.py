@@ -64,3 +64,39 @@ def test_seed_lists_equal_the_oracle(kind, C, W, H, S, leaf, stride, tc):
     np.testing.assert_array_equal(cost.cpu().numpy(), rc)
     ctx.sync()
     ctx.close()
+
+
+def test_allocation_free_search_with_long_tiles():
+    # as many queries as its scratch takes: two chunks, tiles of 512 candidates
+    import torch
+    W = H = 1448
+    f = torch.from_numpy(_frames("smooth", 1, W, H, 4)).cuda()
+    ctx = ff.Context(ff.Config(channels=1, scales=3, iters=1, max_width=W, max_height=H))
+    feat = []
+    for slot in (0, 1):
+        ctx.features(slot, f[slot])
+        x = torch.zeros((H, W, 16), dtype=torch.int8, device="cuda")
+        x[..., :9] = ctx.features_of(slot, 0)
+        feat.append(x)
+    idx, dist = ctx.seed_knn(0)
+    got_i, got_d = torch.empty_like(idx), torch.empty_like(dist)
+    ff.ff_seed_knn_static(feat[0], feat[1], W, H, 1, 3, 8, 1, got_i, got_d,
+                          torch.cuda.current_stream())
+    assert torch.equal(got_i, idx) and torch.equal(got_d, dist)
+    ctx.close()
+
+
+@pytest.mark.parametrize("C,W,H,offset", [(3, 37, 29, 0), (3, 37, 29, 1), (1, 131, 3, 2), (1, 1, 1, 3)])
+def test_feature_read_out_at_any_alignment(C, W, H, offset):
+    import torch
+    f = _frames("noise", C, W, H, 8)
+    ctx = ff.Context(ff.Config(channels=C, scales=1, iters=1, max_width=W, max_height=H))
+    ctx.features(0, torch.from_numpy(f[0]).cuda())
+    buf = torch.full((W * H * 9 * C + 8,), 99, dtype=torch.int8, device="cuda")
+    ff.ff_get_features(ctx.ctx, 0, 0, buf[offset:])
+    got = buf.cpu().numpy()
+    n = W * H * 9 * C
+    np.testing.assert_array_equal(got[offset:offset + n],
+                                  O.features_all(f[0], 1)[0].reshape(-1))
+    assert (got[:offset] == 99).all() and (got[offset + n:] == 99).all()
+    ctx.close()
