@@ -767,7 +767,7 @@ def main():
                     help="choose each batched leg's slots and sweep lane layout by timing "
                          "(autotune.py; the choice is cached)")
     ap.add_argument("--seed-path", choices=["tc", "mma"], default="tc",
-                    help="seeding full pass on tcgen05 (default) or mma.sync")
+                    help="accepted; the seeding search has one path (tcgen05)")
     ap.add_argument("--sweep-lanes", type=int, default=0,
                     help="sweep lanes per grid point (2, 4; 0 = library default)")
     args = ap.parse_args()

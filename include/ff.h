@@ -288,12 +288,12 @@ ff_status ff_sync(ff_ctx *ctx);
  * device-side wait (default 2 s).  FF_DEBUG_FORCE_TIMEOUT: when nonzero, the
  * next propagation sweeps wait for a boundary row that is never written, so
  * the bounded wait runs out and ff_sync reports FF_ETIMEOUT.
- * FF_DEBUG_SWEEP_LANES: lanes of the sweep's propagation warp per grid point,
- * 4 (default: each candidate's cost split over two lanes, 8 rows per strip)
- * or 2 (one lane per candidate, 16 rows per strip: fewer instructions per
- * point, a longer step).  FF_DEBUG_SEED_TC: 1 (default) runs the seeding
- * search's full pass on the tcgen05 tensor cores, 0 on mma.sync.  Every value
- * gives the same results. */
+ * FF_DEBUG_SWEEP_LANES: which sweep kernel runs, 4 (default; 8 means the same:
+ * blocks of four columns, a warp per row, the shortest time for one pair) or 2
+ * (two lanes of a warp per grid point, 16 rows per strip: fewer instructions
+ * per point; what batch and server slots run).  FF_DEBUG_SEED_TC: accepted; the
+ * seeding search has one path, on the tcgen05 tensor cores.  Every value gives
+ * the same results. */
 typedef enum {
     FF_DEBUG_WAIT_LIMIT_NS = 1,
     FF_DEBUG_FORCE_TIMEOUT = 2,

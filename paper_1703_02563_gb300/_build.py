@@ -9,7 +9,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 SOURCES = [os.path.join(CSRC, "ff.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, h) for h in ("ff_kernels.cuh", "ff_sweep.cuh", "ff_block.cuh", "ff_wht_tc.cuh", "ff_seed_tc.cuh",
+DEPS = SOURCES + [os.path.join(CSRC, h) for h in ("ff_kernels.cuh", "ff_sweep.cuh", "ff_block.cuh",
+                                                  "ff_wht_tc.cuh", "ff_seed_tc.cuh",
                                                   "ff_peaks.cuh")] \
     + [os.path.join(ROOT, "include", "ff.h")]
 LIB = os.path.join(HERE, "libff.so")

@@ -221,6 +221,35 @@ __host__ __device__ constexpr size_t block_smem_bytes(int U) {
     return (size_t)kBlkRows * ((U + kBlkCols - 1) / kBlkCols * kBlkCols) * 8;
 }
 
+// One sweep in direction d, after the random search of the sweep before (which
+// only changes a point's own value, so it can be done when the value is fetched).
+//
+// In the sweep's frame (u, v) a point takes the best of its current value, the
+// value above it (u, v-1) and the one to its left (u-1, v), the later in that
+// order on ties: a serial chain.  Here a warp owns a row and decides four columns
+// per step.  A value that reaches column j of a block is the one left of the
+// block, the one above a column i <= j, or the current one of a column i <= j; so
+// 4 + 10 + 10 costs hold every outcome.  Those of current values (the points' own
+// and six "runs" i -> j) do not depend on a neighbour and are staged ahead; the
+// other 14 are evaluated at once, two lanes each, when the row above has decided
+// the block; and the decision is then a chain of compares and selects.
+//
+//  * Row warps 0-3.  Decisions go to the row below as (1 << 32) | flow words: the
+//    next warp's row of shared memory, the next CTA of the cluster's (distributed
+//    shared memory), or, behind a cluster's last row, global memory.
+//  * Stager warps: per block current values after the pending random search, and
+//    the runs' costs; their loads also bring most of what the rows will read into L1.
+//  * Loader warp (first CTA of a cluster): the global row above the cluster.
+// Clusters take their rows in ticket order, so a row only waits for one that runs.
+// Every wait is bounded and warp-uniform, as in the batch sweep.
+//
+// What bounds it: a step of ~1060 cycles (U/4 of them) and a row hand-over of ~870
+// (V of them), both chains of dependent instructions of one warp (about 5 cycles
+// each) with one tap load in them; 57% of the time are the hand-overs.  At 1024x436
+// Lab the level-0 sweep takes 406 us (650 with a step of one column of eight rows,
+// ~920 cycles on each of U + V anti-diagonals).  Two columns per step would double
+// the steps for about a tenth less of a hand-over; eight need 44 costs per step.
+// Four rows per strip keep one row warp on each quarter of an SM.
 template <int C>
 __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_threads(C))
     k_sweep_block(const BlockArgs a) {

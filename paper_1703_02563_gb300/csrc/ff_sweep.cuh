@@ -1,4 +1,5 @@
-// ff_sweep.cuh - propagation sweep + random search kernel (arXiv 1703.02563,
+// ff_sweep.cuh - propagation sweep + random search kernel for many pairs in
+// flight (one pair at a time: ff_block.cuh), and what both share (arXiv 1703.02563,
 // Sec. 3.1 Eq. 2 and the random search step; Sec. 3.2 for R_n = R n).
 #pragma once
 #include "ff_kernels.cuh"
