@@ -1503,11 +1503,11 @@ ff_status ff_features(ff_ctx *c, int slot, const uint8_t *img, int w, int h, int
             dim3 grid((WL + 15) / 16, (HL + 15) / 16);
             prof_begin(c, "k_features");
             if (c->C == 1)
-                k_features_tc<1, false><<<grid, 128, 0, c->stream>>>(img, pitch, w, h, L, WL, HL,
-                                                                     out, nullptr);
+                k_features_tc<1, false><<<grid, tc_feature_threads(L), 0, c->stream>>>(
+                    img, pitch, w, h, L, WL, HL, out, nullptr);
             else
-                k_features_tc<3, false><<<grid, 128, 0, c->stream>>>(img, pitch, w, h, L, WL, HL,
-                                                                     out, nullptr);
+                k_features_tc<3, false><<<grid, tc_feature_threads(L), 0, c->stream>>>(
+                    img, pitch, w, h, L, WL, HL, out, nullptr);
             ff_status s = check_launch(c, "k_features");
             if (s) return s;
         }
@@ -1606,11 +1606,11 @@ ff_status ff_wht_coeffs_tc(const uint8_t *img, int w, int h, int pitch, int chan
     dim3 grid((WL + 15) / 16, (HL + 15) / 16);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (channels == 1)
-        k_features_tc<1, true><<<grid, 128, 0, st>>>(img, pitch, w, h, level, WL, HL, nullptr,
-                                                     coeffs_out);
+        k_features_tc<1, true><<<grid, tc_feature_threads(level), 0, st>>>(
+            img, pitch, w, h, level, WL, HL, nullptr, coeffs_out);
     else
-        k_features_tc<3, true><<<grid, 128, 0, st>>>(img, pitch, w, h, level, WL, HL, nullptr,
-                                                     coeffs_out);
+        k_features_tc<3, true><<<grid, tc_feature_threads(level), 0, st>>>(
+            img, pitch, w, h, level, WL, HL, nullptr, coeffs_out);
     return cudaGetLastError() == cudaSuccess ? FF_OK : FF_ECUDA;
 }
 
@@ -1625,8 +1625,8 @@ ff_status ff_wht_coeffs_scalespace_tc(const uint8_t *img, int w, int h, int pitc
     dim3 grid((WL + 15) / 16, (HL + 15) / 16);
     cudaStream_t st = (cudaStream_t)cuda_stream;
 #define FF_LAUNCH_TCS(CC, IN) \
-    k_features_tc<CC, true, IN><<<grid, 128, 0, st>>>(img, pitch, w, h, level, WL, HL, nullptr, \
-                                                      coeffs_out)
+    k_features_tc<CC, true, IN><<<grid, tc_feature_threads(level), 0, st>>>( \
+        img, pitch, w, h, level, WL, HL, nullptr, coeffs_out)
     if (channels == 1) {
         if (fp16) FF_LAUNCH_TCS(1, 2);
         else FF_LAUNCH_TCS(1, 1);

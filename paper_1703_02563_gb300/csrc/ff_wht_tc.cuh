@@ -64,6 +64,11 @@ __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Threads of a CTA.  Warps 0-3 do the products; from level 2 on, where a tile's
+// averages sum 16 and more pixels each and a level has few tiles, twelve more help
+// to form them (four levels of a 1242x375 Lab frame: 113 -> 84 us).
+__host__ __device__ constexpr int tc_feature_threads(int L) { return L >= 2 ? 512 : 128; }
+
 // One CTA: a 16x16 tile of level pixels, 4 warps x 4 tile rows; each tile
 // row is one m16 fragment (16 pixels), K = 64 in 4 k-steps of two window
 // rows, N = 9 coefficients padded to 16 (two n8 fragments).
@@ -71,7 +76,7 @@ __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)
 // of the int8 features.  IN: 0 the rounded integer level image in bf16; 1,
 // 2 the unrounded FP32 scale-space image rounded to bf16, fp16 (FLOAT_OUT).
 template <int C, bool FLOAT_OUT, int IN = 0>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(tc_feature_threads(FF_MAX_SCALES))
     k_features_tc(const uint8_t *__restrict__ img, int pitch, int W, int H, int L, int WL, int HL,
                   uint8_t *__restrict__ out, float *__restrict__ fout) {
     static_assert(IN == 0 || FLOAT_OUT, "the precision form returns coefficients");
@@ -124,7 +129,7 @@ __global__ void __launch_bounds__(128)
                                               bf16_sign(wht_basis(k0 + 1, col)));
             }
 #pragma unroll 1
-    for (int rr = 0; rr < 4; rr++) {
+    for (int rr = 0; rr < 4 && warp < 4; rr++) {
         const int ty = warp * 4 + rr;
 #pragma unroll
         for (int c = 0; c < C; c++) {
