@@ -5,6 +5,14 @@
 
 namespace ffk {
 
+// Level row that row v of a sweep's frame stands for.  The last strip's and cluster's
+// rows past the frame (v >= V) take the last row's place: their warps form its
+// addresses and load its first query, which they do not use.
+__host__ __device__ constexpr int block_row(int v, int V, bool flipy) {
+    const int r = v < V ? v : V - 1;
+    return flipy ? V - 1 - r : r;
+}
+
 // ---------------------------------------------------------------------------
 // matching error with the query's bytes as they are: per dimension one dp4a
 // seeds the accumulator with -64 q and one adds the four weighted taps
@@ -286,7 +294,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
     } else if (warp < kBlkRows) {
         // ================= a row =================
         const int v = v0 + warp;
-        const int gy = flipy ? V - 1 - v : v;
+        const int gy = block_row(v, V, flipy);
         const int py = gy * n;
         const bool live = v < V, has_v = v > 0;
         // this lane's evaluation: e 0-3 the left value at column e, 4-7 the value
@@ -467,7 +475,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
         const int w = warp - kBlkRows;
         const int r = lane >> 3, i = lane & 3;
         const int v = v0 + r;
-        const int gy = flipy ? V - 1 - v : v;
+        const int gy = block_row(v, V, flipy);
         const int py = gy * n;
         const int loy = -8 * py, hiy = 8 * (H - 1) - 8 * py;
         for (int p = w; 2 * p < NB; p += kStagers) {
