@@ -112,6 +112,11 @@ constexpr int kBlkCluster = 8;               // strips of a cluster
 // the rows for issue slots).
 __host__ __device__ constexpr int blk_stagers(int C) { return C == 3 ? 4 : 2; }
 __host__ __device__ constexpr int blk_threads(int C) { return (kBlkRows + blk_stagers(C) + 1) * 32; }
+// CTAs per SM that the registers have to allow (0: as they come).  Gray: three, i.e. 80
+// registers; with a few more only two fit, which costs 32 contexts on 640x480 frames
+// 13.3 -> 16.6 ms, and with four, 72 registers, a lone 1242x375 pair takes 3.24 ms
+// instead of 3.00.  Lab: two come (96 registers); three spill (1024x436: 8.4 -> 10.8 ms).
+__host__ __device__ constexpr int blk_ctas(int C) { return C == 3 ? 0 : 3; }
 constexpr int kBlkRing = 16;                 // staged blocks per row
 // Levels up to this wide start the next sweep's launch early: its waiting CTAs hold
 // room on the SMs (a 128x96 pair 973 -> 917 us, 1024x436 8.53 -> 8.45 ms; on every
@@ -138,11 +143,15 @@ struct BlockArgs {
 struct BlockStage {
     uint32_t flow[4], cost[4];     // current values, after the pending random search
     uint32_t run[6];               // cost of current flow i at column j: 01 12 23 02 03 13
-    uint32_t tag, pad;             // block + 1, written last
+    uint32_t pad[2];
 };
 
 struct BlockShared {
     BlockStage stage[kBlkRows][kBlkRing];
+    // Block + 1 of each staged block, released last.  Words of their own: a vector load is
+    // a set of loads without an order among them, so one that held a tag and costs could
+    // bring the tag of this block with the costs of the block there before.
+    uint32_t tag[kBlkRows][kBlkRing];
     uint32_t cand[kBlkRows][16];   // costs of a step: H0-3, V0-3, V runs 01 12 23 02 03 13
     int done[kBlkRows];            // blocks each row has finished
     int abort, cluster;
@@ -209,6 +218,16 @@ __device__ __forceinline__ uint4 lds128s(uint32_t p) {
 __device__ __forceinline__ void sts32s(uint32_t p, uint32_t v) {
     asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
 }
+// a flag and what it guards: the writer's lanes meet (__syncwarp) before one of them
+// releases the flag; a reader acquires it before it loads the rest
+__device__ __forceinline__ uint32_t lds32_acquire(uint32_t p) {
+    uint32_t v;
+    asm volatile("ld.acquire.cta.shared::cta.b32 %0, [%1];" : "=r"(v) : "r"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts32_release(uint32_t p, uint32_t v) {
+    asm volatile("st.release.cta.shared::cta.b32 [%0], %1;" ::"r"(p), "r"(v) : "memory");
+}
 __device__ __forceinline__ void launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
@@ -259,7 +278,8 @@ __host__ __device__ constexpr size_t block_smem_bytes(int U) {
 // the steps for about a tenth less of a hand-over; eight need 44 costs per step.
 // Four rows per strip keep one row warp on each quarter of an SM.
 template <int C>
-__global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_threads(C))
+__global__ void __cluster_dims__(kBlkCluster, 1, 1)
+    __launch_bounds__(blk_threads(C), blk_ctas(C))
     k_sweep_block(const BlockArgs a) {
     constexpr int P = Geo<C>::P, LW = P / 8;   // bytes per vector; words of an evaluating lane
     constexpr unsigned FULL = 0xffffffffu;
@@ -274,7 +294,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
     const int NB = (U + kBlkCols - 1) / kBlkCols, UP = NB * kBlkCols;
     const uint32_t rank = cluster_rank();
     for (int j = tid; j < kBlkRows * UP; j += kThreads) vin_all[j] = 0ull;
-    for (int j = tid; j < kBlkRows * kBlkRing; j += kThreads) (&sm.stage[0][0])[j].tag = 0;
+    for (int j = tid; j < kBlkRows * kBlkRing; j += kThreads) (&sm.tag[0][0])[j] = 0;
     if (tid < kBlkRows) sm.done[tid] = 0;
     if (tid == 0) sm.abort = 0;
     if (rank == 0 && tid == 0) sm.cluster = (int)atomicAdd(a.ticket, 1u);
@@ -310,7 +330,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
         // staged blocks, the costs of a step
         uint32_t vin = smem_addr(vin_all + (size_t)warp * UP);
         const uint32_t stage = smem_addr(sm.stage[warp]), cand = smem_addr(sm.cand[warp]);
-        const uint32_t done = smem_addr(&sm.done[warp]);
+        const uint32_t tags = smem_addr(sm.tag[warp]), done = smem_addr(&sm.done[warp]);
         // where the decisions go: the row below, in this CTA or the next of the
         // cluster, or the row in global memory behind the cluster's last strip
         const bool to_cta = warp + 1 < kBlkRows, to_peer = !to_cta && rank + 1 < kBlkCluster;
@@ -357,18 +377,13 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
             uint32_t lo1, hi1, lo2, hi2, lo3, hi3;
             int4 seed[LW];
             auto own_part = [&]() -> bool {
-                cb = lds128s(slot + 48);
-                // not staged yet?  (A vote: a 16-byte load is served in parts, so the lanes
-                // need not see the same tag.)
-                if (!__all_sync(FULL, cb.z == (uint32_t)b + 1)) {
-                    unsigned long long t0 = 0;
-                    for (int k = 1;; k++) {
-                        cb = lds128s(slot + 48);
-                        if (__all_sync(FULL, cb.z == (uint32_t)b + 1)) break;
-                        if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return false;
-                    }
-                }
+                // staged yet?  (A vote: the lanes need not see the same tag.)
+                const uint32_t tag = tags + 4u * (uint32_t)(b & (kBlkRing - 1));
+                unsigned long long t0 = 0;
+                for (int k = 1; !__all_sync(FULL, lds32_acquire(tag) == (uint32_t)b + 1); k++)
+                    if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return false;
                 cf = lds128s(slot), cc = lds128s(slot + 16), ca = lds128s(slot + 32);
+                cb = lds128s(slot + 48);
                 lo1 = add_s16x2(lo0, wstep), hi1 = add_s16x2(hi0, wstep);
                 lo2 = add_s16x2(lo1, wstep), hi2 = add_s16x2(hi1, wstep);
                 lo3 = add_s16x2(lo2, wstep), hi3 = add_s16x2(hi2, wstep);
@@ -520,14 +535,14 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1) __launch_bounds__(blk_thread
                     else rb = s;
                 }
             }
-            BlockStage *st = &sm.stage[r][(2 * p + ((lane >> 2) & 1)) & (kBlkRing - 1)];
+            const int slot = (2 * p + ((lane >> 2) & 1)) & (kBlkRing - 1);
+            BlockStage *st = &sm.stage[r][slot];
             st->flow[i] = f;
             st->cost[i] = c;
             st->run[i] = ra;
             if (i < 2) st->run[4 + i] = rb;
-            __threadfence_block();
             __syncwarp();
-            if (i == 0) sts32s(smem_addr(&st->tag), (uint32_t)(u >> 2) + 1);
+            if (i == 0) sts32_release(smem_addr(&sm.tag[r][slot]), (uint32_t)(u >> 2) + 1);
         }
     } else if (rank == 0 && strip > 0) {
         // ================= the loader: the row above this cluster =================

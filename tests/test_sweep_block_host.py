@@ -35,11 +35,32 @@ int main() {
 """
 
 
-def test_every_row_of_a_strip_is_a_row_of_the_level(tmp_path):
-    src, exe = tmp_path / "rows.cu", tmp_path / "rows"
-    src.write_text(ROWS)
+# A vector load has no order among its words: a tag must not share one with what it stands for.
+TAGS = r"""
+#include <cstddef>
+#include "ff_block.cuh"
+int main() {
+    using namespace ffk;
+    const size_t stage = offsetof(BlockShared, stage), tag = offsetof(BlockShared, tag);
+    const size_t end = stage + sizeof(BlockShared::stage);
+    return sizeof(BlockStage) % 16 || stage % 16 || !(tag >= (end + 15) / 16 * 16 || tag < stage);
+}
+"""
+
+
+def _run(text, tmp_path):
+    src, exe = tmp_path / "check.cu", tmp_path / "check"
+    src.write_text(text)
     inc = os.path.join(_build.ROOT, "include")
     subprocess.run([_build.nvcc(), *_build.ARCH, "-std=c++17", "-I", _build.CSRC, "-I", inc,
                     "-o", str(exe), str(src)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
+
+
+def test_every_row_of_a_strip_is_a_row_of_the_level(tmp_path):
+    _run(ROWS, tmp_path)
+
+
+def test_staged_tags_share_no_vector_with_the_staged_values(tmp_path):
+    _run(TAGS, tmp_path)
