@@ -248,6 +248,18 @@ __host__ __device__ constexpr size_t block_smem_bytes(int U) {
     return (size_t)kBlkRows * ((U + kBlkCols - 1) / kBlkCols * kBlkCols) * 8;
 }
 
+// Poll k of a wait that found nothing; true when the warp must give up.  Every 64th looks
+// at the clock and the CTA's abort flag, every 1024th (about 20 us) also whether another
+// CTA or an earlier sweep of this direction has given up, so that one expiry ends the
+// whole match: a load from global memory, which at every look would hold up the hand-over
+// that is waited for.
+__device__ __forceinline__ bool wait_over(int k, unsigned long long &t0, unsigned long long wait_ns,
+                                          volatile int *abort_flag, int *err) {
+    if (k & 63) return false;
+    if ((k & 1023) == 0 && ld_relaxed_i32(err) != 0) *abort_flag = 1;
+    return wait_expired(t0, wait_ns, abort_flag, err);
+}
+
 // One sweep in direction d, after the random search of the sweep before (which
 // only changes a point's own value, so it can be done when the value is fetched).
 //
@@ -268,7 +280,8 @@ __host__ __device__ constexpr size_t block_smem_bytes(int U) {
 //    the runs' costs; their loads also bring most of what the rows will read into L1.
 //  * Loader warp (first CTA of a cluster): the global row above the cluster.
 // Clusters take their rows in ticket order, so a row only waits for one that runs.
-// Every wait is bounded and warp-uniform, as in the batch sweep.
+// Every wait is bounded and warp-uniform, and one that expires ends the others, as in
+// the batch sweep.
 //
 // What bounds it: a step of ~1060 cycles (U/4 of them) and a row hand-over of ~870
 // (V of them), both chains of dependent instructions of one warp (about 5 cycles
@@ -381,7 +394,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
                 const uint32_t tag = tags + 4u * (uint32_t)(b & (kBlkRing - 1));
                 unsigned long long t0 = 0;
                 for (int k = 1; !__all_sync(FULL, lds32_acquire(tag) == (uint32_t)b + 1); k++)
-                    if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) return false;
+                    if (wait_over(k, t0, a.wait_ns, v_abort, a.err)) return false;
                 cf = lds128s(slot), cc = lds128s(slot + 16), ca = lds128s(slot + 32);
                 cb = lds128s(slot + 48);
                 lo1 = add_s16x2(lo0, wstep), hi1 = add_s16x2(hi0, wstep);
@@ -403,7 +416,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
                 for (int k = 1;; k++) {
                     va = lds64s(vin + 8 * src);
                     if (__all_sync(FULL, (uint32_t)(va >> 32) == want)) break;
-                    if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) goto finished;
+                    if (wait_over(k, t0, a.wait_ns, v_abort, a.err)) goto finished;
                 }
             }
             // this lane's candidate, clamped into the frame; its taps and weights
@@ -501,7 +514,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
                 const bool ok = lane >= kBlkRows ||
                                 (int)lds32s(smem_addr(&sm.done[lane])) + kBlkRing >= 2 * p + 2;
                 if (__all_sync(FULL, ok)) break;
-                if ((k & 63) == 0 && wait_expired(t0, a.wait_ns, v_abort, a.err)) goto finished;
+                if (wait_over(k, t0, a.wait_ns, v_abort, a.err)) goto finished;
             }
             if (p == 0) launch_dependents();   // (the next sweep's launch may come in)
             const int u = 8 * p + (lane & 7);
@@ -547,7 +560,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
     } else if (rank == 0 && strip > 0) {
         // ================= the loader: the row above this cluster =================
         const unsigned long long *srow = a.edge + (size_t)(cluster - 1) * U;
-        int base = 0;
+        int base = 0, k = 0;
         unsigned long long t0 = 0;
         while (base < U) {
             const int col = base + lane;
@@ -562,7 +575,8 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             if (got > 0) {
                 base += got;
                 t0 = 0;
-            } else if (wait_expired(t0, a.wait_ns, v_abort, a.err)) {
+                k = 0;
+            } else if (wait_over(++k, t0, a.wait_ns, v_abort, a.err)) {
                 break;
             }
         }

@@ -81,3 +81,34 @@ def test_block_and_batch_sweeps_agree_on_large_frames(schedule):
             np.testing.assert_array_equal(a, b)
     ctx.sync()
     ctx.close()
+
+
+# one expired wait ends the match: its other CTAs (of the tall frame not all fit the GPU at
+# once) and its later sweeps do not wait for their own limit
+@pytest.mark.parametrize("C,W,H,S", [(1, 128, 96, 3), (3, 128, 96, 3), (1, 64, 4096, 1)])
+def test_an_expired_wait_ends_the_match(C, W, H, S):
+    import time
+
+    import torch
+    limit = 0.25
+    pair = workloads.random_pair(seed=C, width=W, height=H, channels=C)
+    ctx = ff.Context(ff.Config(channels=C, scales=S, iters=4, seed_stride=8, max_width=W,
+                               max_height=H))
+    want = _run(ctx, pair, 1)
+    ctx.sync()
+    ff.ff_debug_set(ctx.ctx, ff.FF_DEBUG_WAIT_LIMIT_NS, int(limit * 1e9))
+    ff.ff_debug_set(ctx.ctx, ff.FF_DEBUG_FORCE_TIMEOUT, 1)
+    torch.cuda.synchronize()
+    start = time.perf_counter()
+    ctx.match(0, 1)
+    with pytest.raises(ff.FFError) as e:
+        ctx.sync()
+    took = time.perf_counter() - start
+    assert e.value.status == ff.FF_ETIMEOUT
+    assert limit <= took < 2 * limit
+    ff.ff_debug_set(ctx.ctx, ff.FF_DEBUG_FORCE_TIMEOUT, 0)
+    for a, b in zip(_run(ctx, pair, 1), want):
+        for x, y in zip(a, b):
+            np.testing.assert_array_equal(x, y)
+    ctx.sync()
+    ctx.close()
