@@ -384,13 +384,23 @@ struct KnnOut {
     uint32_t *flow;                // [queries], or NULL
     int *cost;
 };
+// An int where a caller's array has it: the array may start at any byte.
+__device__ __forceinline__ void store_any(int *p, int v) {
+    if (((uintptr_t)p & 3) == 0) {
+        *p = v;
+    } else {
+        uint8_t *b = reinterpret_cast<uint8_t *>(p);
+#pragma unroll
+        for (int k = 0; k < 4; k++) b[k] = (uint8_t)((uint32_t)v >> (8 * k));
+    }
+}
 template <int C>
 __device__ __forceinline__ void knn_finish(const KnnOut &o, int q, int lane, KnnList l) {
     constexpr int P = Geo<C>::P;
     const bool ok = lane < o.leaf && l.D != 0x7fffffff;
     if (o.idx && lane < o.leaf) {
-        o.idx[(size_t)q * o.leaf + lane] = ok ? l.I : -1;
-        o.dist[(size_t)q * o.leaf + lane] = ok ? l.D : -1;
+        store_any(o.idx + (size_t)q * o.leaf + lane, ok ? l.I : -1);
+        store_any(o.dist + (size_t)q * o.leaf + lane, ok ? l.D : -1);
     }
     if (!o.flow) return;
     const int gy = q / o.WL, gx = q - gy * o.WL;

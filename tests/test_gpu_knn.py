@@ -100,3 +100,23 @@ def test_feature_read_out_at_any_alignment(C, W, H, offset):
                                   O.features_all(f[0], 1)[0].reshape(-1))
     assert (got[:offset] == 99).all() and (got[offset + n:] == 99).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_search_writes_arrays_at_any_alignment(offset):
+    import torch
+    W, H, leaf = 61, 43, 5
+    f = torch.from_numpy(_frames("smooth", 3, W, H, 6)).cuda()
+    ctx = ff.Context(ff.Config(channels=3, scales=2, iters=1, seed_leaf=leaf, max_width=W,
+                               max_height=H))
+    for slot in (0, 1):
+        ctx.features(slot, f[slot])
+    want = ctx.seed_knn(0)
+    n = want[0].numel() * 4
+    buf = torch.full((2, n + 16), 99, dtype=torch.uint8, device="cuda")
+    ff.ff_seed_knn(ctx.ctx, 0, buf[0].data_ptr() + offset, buf[1].data_ptr() + 4 + offset)
+    ctx.sync()
+    for row, o, w in zip(buf.cpu().numpy(), (offset, 4 + offset), want):
+        np.testing.assert_array_equal(row[o:o + n], w.cpu().numpy().reshape(-1).view(np.uint8))
+        assert (row[:o] == 99).all() and (row[o + n:] == 99).all()
+    ctx.close()
