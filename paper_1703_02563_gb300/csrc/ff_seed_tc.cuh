@@ -131,6 +131,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *m, uint32_t parity, unsigned
     }
     return true;
 }
+// The same for a whole warp, with one answer for all its lanes: what follows (the
+// tensor-memory loads) takes every lane or none.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *m, uint32_t parity,
+                                               unsigned long long wait_ns,
+                                               volatile int *abort_flag, int *err) {
+    if (__all_sync(0xffffffffu, mbar_test(m, parity))) return true;
+    const unsigned long long t0 = globaltimer_ns();
+    while (!__all_sync(0xffffffffu, mbar_test(m, parity))) {
+        int stop = *abort_flag;
+        if (!stop && globaltimer_ns() - t0 > wait_ns) {
+            atomicCAS(err, 0, kErrTimeout);
+            *abort_flag = 1;
+            stop = 1;
+        }
+        if (__any_sync(0xffffffffu, stop)) return false;
+    }
+    return true;
+}
+// After giving up: the phase, abort or not, for a second at most.
+__device__ __forceinline__ void mbar_drain(uint64_t *m, uint32_t parity) {
+    const unsigned long long t0 = globaltimer_ns();
+    while (!mbar_test(m, parity) && globaltimer_ns() - t0 < 1000000000ull) {
+    }
+}
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *m, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc_smem(m)),
                  "r"(bytes)
@@ -199,7 +223,8 @@ __device__ __forceinline__ float tmem_min128(uint32_t taddr) {
 // and issues the K/16 MMAs of a tile once its accumulator has been drained.
 // Each thread of the epilogue warps (0-3) takes its row's least key out of the
 // accumulator with one reducing tensor-memory load and puts (least key, tile)
-// into its list of eight.  All waits are bounded.  The list of chunk c and
+// into its list of eight.  All waits are bounded; an issuing thread that gives up waits
+// (bounded too) for its copies and products under way.  The list of chunk c and
 // query row q is lists[(c * 128 nqt + q) * 8 ..], empty entries 0xffffffff.
 template <int KS>
 __global__ void __launch_bounds__(192, 2)
@@ -255,14 +280,16 @@ __global__ void __launch_bounds__(192, 2)
                 mbar_expect_tx(&bar_a, TILE_BYTES);
                 bulk_copy(sA, qtile + (size_t)qt * TILE_BYTES, TILE_BYTES, &bar_a);
             }
-            for (int n = 0; n < min(kTcStages, mine); n++) copy(n);
+            int sent = 0;          // copies so far; products so far: n
+            while (sent < min(kTcStages, mine)) copy(sent++);
             // kind::f16, bf16 x bf16 -> f32, both K-major, N = 128, M = 128
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
                                        ((uint32_t)(kTcRows >> 3) << 17) |
                                        ((uint32_t)(kTcRows >> 4) << 24);
             const uint32_t d = taddr + (uint32_t)(g * kTcRows);
             const bool have_a = mbar_wait(&bar_a, 0, wait_ns, v_abort, err);
-            for (int n = 0; n < mine && have_a; n++) {
+            int n = 0;
+            for (; n < mine && have_a; n++) {
                 const int s = n % kTcStages;
                 if (!mbar_wait(&fullg[s], (n / kTcStages) & 1, wait_ns, v_abort, err)) break;
                 if (n >= 1 && !mbar_wait(&acce[g], (n - 1) & 1, wait_ns, v_abort, err)) break;
@@ -281,7 +308,13 @@ __global__ void __launch_bounds__(192, 2)
                         "r"(tc_smem(&accf[g]))
                     : "memory");
                 // tile n - 1 has been drained, so its product is done with its stage
-                if (n >= 1 && n - 1 + kTcStages < mine) copy(n - 1 + kTcStages);
+                if (n >= 1 && sent < mine) copy(sent++);
+            }
+            if (n < mine) {
+                // gave up: no copy or product may still be under way when the CTA ends
+                if (g == 0) mbar_drain(&bar_a, 0);
+                for (int m = n; m < sent; m++) mbar_drain(&fullg[m % kTcStages], (m / kTcStages) & 1);
+                if (n > 0) mbar_drain(&accf[g], (n - 1) & 1);
             }
         }
     } else {
@@ -293,7 +326,7 @@ __global__ void __launch_bounds__(192, 2)
         for (int e = 0; e < 8; e++) l[e] = 0xffffffffu;
         for (int t = 0; t < ntiles; t++) {
             const int g = t & 1;
-            if (!mbar_wait(&accf[g], (t >> 1) & 1, wait_ns, v_abort, err)) break;
+            if (!mbar_wait_warp(&accf[g], (t >> 1) & 1, wait_ns, v_abort, err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const float least = tmem_min128(ta + (uint32_t)(g * kTcRows));
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

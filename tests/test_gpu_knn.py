@@ -120,3 +120,28 @@ def test_search_writes_arrays_at_any_alignment(offset):
         np.testing.assert_array_equal(row[o:o + n], w.cpu().numpy().reshape(-1).view(np.uint8))
         assert (row[:o] == 99).all() and (row[o + n:] == 99).all()
     ctx.close()
+
+
+@pytest.mark.parametrize("C,S", [(1, 4), (3, 2)])
+def test_search_with_the_shortest_wait_limit_ends_and_recovers(C, S):
+    # whether a wait runs out is up to the load: each search either reports it or is right,
+    # and the next one with the usual limit is right
+    import torch
+    W, H = 640, 200
+    f = torch.from_numpy(_frames("smooth", C, W, H, 9)).cuda()
+    ctx = ff.Context(ff.Config(channels=C, scales=S, iters=1, max_width=W, max_height=H))
+    for slot in (0, 1):
+        ctx.features(slot, f[slot])
+    want = ctx.seed_knn(0)
+    ctx.sync()
+    for limit in (1000, 1000, 1000, 2_000_000_000):
+        ff.ff_debug_set(ctx.ctx, ff.FF_DEBUG_WAIT_LIMIT_NS, limit)
+        got = ctx.seed_knn(0)
+        try:
+            ctx.sync()
+        except ff.FFError as e:
+            assert e.status == ff.FF_ETIMEOUT and limit == 1000
+            continue
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
+    ctx.close()
