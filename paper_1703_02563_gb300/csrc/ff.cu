@@ -153,12 +153,13 @@ __global__ void __launch_bounds__(128)
 // dimensions -- for k_seed_pick to rank (ff_seed_tc.cuh has the argument), but
 // without tiles of its own in memory: QPT queries per thread, one chunk of tiles per
 // blockIdx.y, 128 candidates at a time staged in shared memory with their norms in
-// the row's free last word.  A tile has `trows` candidates, a multiple of 128.
+// the row's free last word.  A tile has `trows` candidates: 32 (FINE, where there are few
+// candidates: kTcFineTiles), or a multiple of 128.
 //
 // What bounds it: the dp4a and minimum per candidate and query (exact lists of
 // candidates, kept here before, took their insertion path for most candidates
 // of a warp: 605 us at 640x480 gray, every second candidate).
-template <int C, int QPT>
+template <int C, int QPT, bool FINE>
 __global__ void __launch_bounds__(128)
     k_seed_scan(const uint8_t *__restrict__ f1, const uint8_t *__restrict__ f2, int W, int N,
                 int WS, int NQ, int stride, int Wc, int ncand, int trows, int chunk,
@@ -209,35 +210,40 @@ __global__ void __launch_bounds__(128)
             for (int v = 0; v < NV; v++) s_w[threadIdx.x][v] = r[v];
         }
         __syncthreads();
+        auto scan = [&](int k0, int k1) {
 #pragma unroll 4
-        for (int k = 0; k < kTcRows; k++) {
-            uint32_t cw[NV * 4];
+            for (int k = k0; k < k1; k++) {
+                uint32_t cw[NV * 4];
 #pragma unroll
-            for (int v = 0; v < NV; v++) {
-                const uint4 x = s_w[k][v];
-                cw[4 * v] = x.x, cw[4 * v + 1] = x.y, cw[4 * v + 2] = x.z, cw[4 * v + 3] = x.w;
-            }
-#pragma unroll
-            for (int j = 0; j < QPT; j++) {
-                int dot = 0;
-#pragma unroll
-                for (int w = 0; w < NW; w++) dot = __dp4a((int)qw[j][w], (int)cw[w], dot);
-                least[j] = min(least[j], (int)cw[NV * 4 - 1] - 2 * dot);
-            }
-        }
-        if ((base + kTcRows - c0) % trows == 0 || base + kTcRows >= c1) {   // a tile ends
-            const uint32_t t = (uint32_t)((base - c0) / trows);
-#pragma unroll
-            for (int j = 0; j < QPT; j++) {
-                uint32_t x = ((uint32_t)(least[j] + kTcKeyBias) << kTcTileBits) + t;
-#pragma unroll
-                for (int e = 0; e < 8; e++) {
-                    const uint32_t lo = min(l[j][e], x);
-                    x = max(l[j][e], x);
-                    l[j][e] = lo;
+                for (int v = 0; v < NV; v++) {
+                    const uint4 x = s_w[k][v];
+                    cw[4 * v] = x.x, cw[4 * v + 1] = x.y, cw[4 * v + 2] = x.z, cw[4 * v + 3] = x.w;
                 }
+#pragma unroll
+                for (int j = 0; j < QPT; j++) {
+                    int dot = 0;
+#pragma unroll
+                    for (int w = 0; w < NW; w++) dot = __dp4a((int)qw[j][w], (int)cw[w], dot);
+                    least[j] = min(least[j], (int)cw[NV * 4 - 1] - 2 * dot);
+                }
+            }
+        };
+        auto tile_ends = [&](uint32_t t) {
+#pragma unroll
+            for (int j = 0; j < QPT; j++) {
+                tile_insert(l[j], ((uint32_t)(least[j] + kTcKeyBias) << kTcTileBits) + t);
                 least[j] = kMissing;
             }
+        };
+        if constexpr (FINE) {
+            for (int k = 0; k < kTcRows && base + k < c1; k += kTcFineRows) {
+                scan(k, k + kTcFineRows);
+                tile_ends((uint32_t)((base + k - c0) / kTcFineRows));
+            }
+        } else {
+            scan(0, kTcRows);
+            if ((base + kTcRows - c0) % trows == 0 || base + kTcRows >= c1)
+                tile_ends((uint32_t)((base - c0) / trows));
         }
     }
 #pragma unroll
@@ -855,12 +861,17 @@ ff_status launch_seed(ff_ctx *c, int d, const uint8_t *fs, const uint8_t *fd, in
                                                              ncand, st.qtile, st.ctile);
     if ((s = check_launch(c, "k_seed_prep"))) return s;
     prof_begin(c, "k_seed_scan");
-    k_seed_tc<KS><<<dim3(z.nqt, z.nch), 192, tc_seed_smem_bytes<KS>(), c->stream>>>(
+    const dim3 grid(z.nqt, z.nch);
+    const bool fine = z.nct <= kTcFineTiles;
+    (fine ? k_seed_tc<KS, true> : k_seed_tc<KS, false>)<<<grid, 192, tc_seed_smem_bytes<KS>(),
+                                                         c->stream>>>(
         st.qtile, st.ctile, z.nct, z.chunk, st.lists, st.err, c->wait_ns);
     if ((s = check_launch(c, "k_seed_scan"))) return s;
     prof_begin(c, "k_seed_merge");
-    k_seed_pick<C><<<(nq + 3) / 4, 128, 0, c->stream>>>(fs, fd, W, N, WS, nq, stride, Wc, ncand,
-                                                        st.lists, z.nqt, z.nch, z.chunk, kTcRows, out);
+    const int trows = fine ? kTcFineRows : kTcRows;
+    (fine ? k_seed_pick<C, true> : k_seed_pick<C, false>)<<<(nq + 3) / 4, 128, 0, c->stream>>>(
+        fs, fd, W, N, WS, nq, stride, Wc, ncand, st.lists, z.nqt, z.nch,
+        z.chunk * (kTcRows / trows), trows, out);
     return check_launch(c, "k_seed_merge");
 }
 
@@ -1403,9 +1414,13 @@ ff_status ff_create(const ff_config *cfg, int device, void *cuda_stream, ff_ctx 
     if (cudaGetDeviceCount(&ndev) != cudaSuccess || device < 0 || device >= ndev) return FF_ECUDA;
     DeviceGuard guard(device);
     // these take more than 48 KB of shared memory (the sweep: on wide frames)
-    if (cudaFuncSetAttribute(k_seed_tc<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(k_seed_tc<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc_seed_smem_bytes<1>()) != cudaSuccess ||
-        cudaFuncSetAttribute(k_seed_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_seed_tc<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc_seed_smem_bytes<1>()) != cudaSuccess ||
+        cudaFuncSetAttribute(k_seed_tc<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             tc_seed_smem_bytes<2>()) != cudaSuccess ||
+        cudaFuncSetAttribute(k_seed_tc<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              tc_seed_smem_bytes<2>()) != cudaSuccess ||
         cudaFuncSetAttribute(k_sweep_block<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)block_smem_bytes(FF_MAX_DIM)) != cudaSuccess ||
@@ -1780,13 +1795,15 @@ ff_status ff_seed_knn_static(const int8_t *feat_src0, const int8_t *feat_dst0, i
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
         return *msg = "device query failed", FF_ECUDA;
     // chunks for about kCtasPerSm CTAs per SM, as far as their lists fit the scratch;
-    // tiles long enough that a chunk's have numbers of kTcTileBits
+    // fine tiles for few candidates, else tiles long enough that a chunk's have numbers of
+    // kTcTileBits
     const int nqt = ((int)nq + kTcRows - 1) / kTcRows, nqpad = nqt * kTcRows;
     const int qt = ((int)nq + kSeedQueriesPerCta - 1) / kSeedQueriesPerCta;
     const int cap = (int)(kStaticScratchInt2 * 2 / 8 / (size_t)nqpad);   // >= 1: nq is limited
     const int rows = (ncand + kTcRows - 1) / kTcRows;
     const int want = max(1, min(min(kCtasPerSm * sms / qt, cap), rows));
-    int trows = kTcRows;
+    const bool fine = rows <= kTcFineTiles;
+    int trows = fine ? kTcFineRows : kTcRows;
     while ((long long)trows * want * kTcChunkTiles < ncand) trows *= 2;
     const int tiles = (ncand + trows - 1) / trows;
     const int chunk = (tiles + want - 1) / want, nch = (tiles + chunk - 1) / chunk;
@@ -1794,24 +1811,19 @@ ff_status ff_seed_knn_static(const int8_t *feat_src0, const int8_t *feat_dst0, i
     const uint8_t *fs = (const uint8_t *)feat_src0, *fd = (const uint8_t *)feat_dst0;
     uint32_t *lists = (uint32_t *)scratch;
     const dim3 grid((unsigned)qt, nch);
-    if (channels == 1)
-        k_seed_scan<1, kSeedQpt><<<grid, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc,
-                                                          ncand, trows, chunk, lists, nqpad);
-    else
-        k_seed_scan<3, kSeedQpt><<<grid, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc,
-                                                          ncand, trows, chunk, lists, nqpad);
+    (channels == 1 ? (fine ? k_seed_scan<1, kSeedQpt, true> : k_seed_scan<1, kSeedQpt, false>)
+                   : (fine ? k_seed_scan<3, kSeedQpt, true> : k_seed_scan<3, kSeedQpt, false>))
+        <<<grid, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand, trows, chunk,
+                                   lists, nqpad);
     if (cudaGetLastError() != cudaSuccess) return *msg = "k_seed_scan launch failed", FF_ECUDA;
     KnnOut out{};
     out.leaf = leaf;
     out.idx = idx_out;
     out.dist = dist_out;
-    const unsigned nb = (unsigned)((nq + 3) / 4);
-    if (channels == 1)
-        k_seed_pick<1><<<nb, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand, lists,
-                                               nqt, nch, chunk, trows, out);
-    else
-        k_seed_pick<3><<<nb, 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand, lists,
-                                               nqt, nch, chunk, trows, out);
+    (channels == 1 ? (fine ? k_seed_pick<1, true> : k_seed_pick<1, false>)
+                   : (fine ? k_seed_pick<3, true> : k_seed_pick<3, false>))
+        <<<(unsigned)((nq + 3) / 4), 128, 0, stream>>>(fs, fd, w, N, WS, (int)nq, stride, Wc, ncand,
+                                                       lists, nqt, nch, chunk, trows, out);
     if (cudaGetLastError() != cudaSuccess) return *msg = "k_seed_pick launch failed", FF_ECUDA;
     return FF_OK;
 }

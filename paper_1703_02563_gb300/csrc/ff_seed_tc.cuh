@@ -35,6 +35,15 @@ constexpr int kTcStages = 4;    // candidate tiles in flight per accumulator
 constexpr int kTcKeyBias = 27 * 128 * 128;
 constexpr int kTcTileBits = 11;
 constexpr int kTcChunkTiles = 1 << kTcTileBits;   // tiles of a chunk, at most
+// Up to this many tiles of candidates the lists keep tiles of 32 candidates instead of
+// 128.  Ranking 8 x 128 is then most of a search (19200 queries, 1200 candidates, Lab: 165 us;
+// 70 with tiles of 32, which is 0.3 to 1.0 of the time at 10 to 235 tiles), while the
+// product, whose epilogue inserts four times as often, takes over with more of them (0.95
+// of the time on average at 294 tiles, 1.03 at 509).
+constexpr int kTcFineTiles = 256;
+constexpr int kTcFineRows = 32;
+static_assert(kTcFineTiles * (kTcRows / kTcFineRows) <= kTcChunkTiles, "fine tiles of a chunk");
+constexpr int kTcMaxKey = 3 * 27 * 128 * 128;     // no candidate's key is above it
 
 // Byte offset of element (r, k) in a tile of 128 rows x K bf16 laid out for
 // the tensor core without swizzling: 8-row x 16-byte core matrices, the K
@@ -216,6 +225,38 @@ __device__ __forceinline__ float tmem_min128(uint32_t taddr) {
     return __uint_as_float(least);
 }
 
+// The same for each 32 of the 128 columns: four loads, one wait.
+#define FF_T8(d) "t" #d "0, t" #d "1, t" #d "2, t" #d "3, t" #d "4, t" #d "5, t" #d "6, t" #d "7"
+#define FF_LD_MIN32(out, a, b, c, d, addr)                                                      \
+    "tcgen05.ld.red.sync.aligned.32x32b.x32.min.f32 {" FF_T8(a) ", " FF_T8(b) ", " FF_T8(c)     \
+    ", " FF_T8(d) "}, " out ", [" addr "];\n\t"
+__device__ __forceinline__ void tmem_min32(uint32_t taddr, float (&least)[4]) {
+    uint32_t m[4];
+    asm volatile("{\n\t.reg .b32 t<170>;\n\t"
+                 FF_LD_MIN32("%0", 1, 2, 3, 4, "%4")
+                 FF_LD_MIN32("%1", 5, 6, 7, 8, "%5")
+                 FF_LD_MIN32("%2", 9, 10, 11, 12, "%6")
+                 FF_LD_MIN32("%3", 13, 14, 15, 16, "%7")
+                 "tcgen05.wait::ld.sync.aligned;\n\t}"
+                 : "=r"(m[0]), "=r"(m[1]), "=r"(m[2]), "=r"(m[3])
+                 : "r"(taddr), "r"(taddr + 32), "r"(taddr + 64), "r"(taddr + 96)
+                 : "memory");
+#pragma unroll
+    for (int s = 0; s < 4; s++) least[s] = __uint_as_float(m[s]);
+}
+#undef FF_LD_MIN32
+#undef FF_T8
+
+// (least key, tile) into a thread's list of eight
+__device__ __forceinline__ void tile_insert(uint32_t (&l)[8], uint32_t x) {
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        const uint32_t lo = min(l[e], x);
+        x = max(l[e], x);
+        l[e] = lo;
+    }
+}
+
 // Per CTA: 128 queries (tensor-memory lanes; epilogue thread = query row)
 // against one chunk of candidates, 128 per tile; even tiles go through one
 // 128-column accumulator, odd ones through the other, and each has its own
@@ -226,7 +267,11 @@ __device__ __forceinline__ float tmem_min128(uint32_t taddr) {
 // into its list of eight.  All waits are bounded; an issuing thread that gives up waits
 // (bounded too) for its copies and products under way.  The list of chunk c and
 // query row q is lists[(c * 128 nqt + q) * 8 ..], empty entries 0xffffffff.
-template <int KS>
+//
+// FINE: the lists' tiles have 32 candidates (tiles 4 t .. 4 t + 3 of a chunk are the
+// product's tile t), so that k_seed_pick has a quarter of the candidates to rank, for four
+// insertions per product here.
+template <int KS, bool FINE>
 __global__ void __launch_bounds__(192, 2)
     k_seed_tc(const uint8_t *__restrict__ qtile, const uint8_t *__restrict__ ctile, int nct,
               int chunk, uint32_t *__restrict__ lists, int *err, unsigned long long wait_ns) {
@@ -328,18 +373,20 @@ __global__ void __launch_bounds__(192, 2)
             const int g = t & 1;
             if (!mbar_wait_warp(&accf[g], (t >> 1) & 1, wait_ns, v_abort, err)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const float least = tmem_min128(ta + (uint32_t)(g * kTcRows));
+            constexpr int F = FINE ? 4 : 1;
+            float least[4];
+            if constexpr (FINE) tmem_min32(ta + (uint32_t)(g * kTcRows), least);
+            else least[0] = tmem_min128(ta + (uint32_t)(g * kTcRows));
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&acce[g]);
-            // key + bias in the low mantissa bits of 2^23 + key + bias (exact)
-            uint32_t x = (__float_as_uint(least + (float)(8388608 + kTcKeyBias)) << kTcTileBits) +
-                         (uint32_t)t;
 #pragma unroll
-            for (int e = 0; e < 8; e++) {
-                const uint32_t lo = min(l[e], x);
-                x = max(l[e], x);
-                l[e] = lo;
+            for (int f = 0; f < F; f++) {
+                // key + bias in the low mantissa bits of 2^23 + key + bias (exact).  A fine
+                // tile may be all padding (+inf): a key above every other stands for it.
+                const float key = FINE ? fminf(least[f], (float)(kTcMaxKey + 1)) : least[f];
+                tile_insert(l, (__float_as_uint(key + (float)(8388608 + kTcKeyBias)) << kTcTileBits) +
+                                   (uint32_t)(F * t + f));
             }
         }
         const size_t row = ((size_t)blockIdx.y * gridDim.x + qt) * kTcRows + warp * 32 + lane;
@@ -460,9 +507,14 @@ __device__ __forceinline__ void knn_finish(const KnnOut &o, int q, int lane, Knn
 // A query's tile lists -> its top 8 (and, for a match, its coarsest flow); one
 // warp per query.  The eight tiles of least (key, tile) come from its nch
 // lists; the eighth's least key bounds the eighth distance, so few of their
-// candidates (8 x 128 from the tensor cores) are kept: those are collected and
-// sorted once.  A tile has `trows` candidates, a multiple of 128.
-template <int C>
+// candidates are kept: those are collected and sorted once.  A tile has `trows`
+// candidates: 32 (FINE), or a multiple of 128.
+//
+// What bounds it: the tiles' rows through L1, where rows a stride apart are lines of their
+// own (8 x 128 of them per query, 19200 queries, Lab: 61 us with every pixel a candidate,
+// 157 us with every eighth; 8 x 32: 53 us).  Halves of a row by a pair of lanes took 44 us
+// there but 72 instead of 62 with every pixel.
+template <int C, bool FINE>
 __global__ void __launch_bounds__(128)
     k_seed_pick(const uint8_t *__restrict__ fq, const uint8_t *__restrict__ fc, int W, int N,
                 int WS, int nq, int stride, int Wc, int ncand, const uint32_t *__restrict__ lists,
@@ -509,15 +561,24 @@ __global__ void __launch_bounds__(128)
     int bD = D7 == 0x7fffffff ? D7 : D7 - kTcKeyBias + qn, bI = 0x7fffffff;
     KnnList l{0x7fffffff, 0x7fffffff};
     int held = 0;                  // candidates in buf, all before (bD, bI) when they came
-    for (int k = 0; k < 8; k++) {
+    // 128 candidates at a time: a stretch of a tile, or four fine tiles
+    for (int k = 0; k < 8; k += FINE ? 4 : 1) {
         const int t = __shfl_sync(FULL, best.I, k);
         if (t == 0x7fffffff) break;
-        for (int o0 = t * trows; o0 < min((t + 1) * trows, ncand); o0 += kTcRows) {
+        const int end = FINE ? t * trows + 1 : min((t + 1) * trows, ncand);
+        for (int o0 = t * trows; o0 < end; o0 += kTcRows) {
             uint4 r[4][NV];
             int idx[4];
+            bool in[4];
 #pragma unroll
             for (int j = 0; j < 4; j++) {
-                idx[j] = min(o0 + 32 * j + lane, ncand - 1);
+                int c = o0 + 32 * j + lane;
+                if (FINE) {
+                    const int tj = __shfl_sync(FULL, best.I, k + j);
+                    c = tj == 0x7fffffff ? ncand : tj * kTcFineRows + lane;
+                }
+                in[j] = c < ncand;
+                idx[j] = min(c, ncand - 1);
                 if (stride > 1) {
                     const int cy = idx[j] / Wc, cx = idx[j] - cy * Wc;
                     idx[j] = cy * stride * W + cx * stride;
@@ -536,7 +597,7 @@ __global__ void __launch_bounds__(128)
                     nn = __dp4a((int)cw, (int)cw, nn);
                 }
                 const int d = nn + qn - 2 * dot;
-                const bool hit = o0 + 32 * j + lane < ncand && lex_less(d, idx[j], bD, bI);
+                const bool hit = in[j] && lex_less(d, idx[j], bD, bI);
                 const unsigned m = __ballot_sync(FULL, hit);
                 if (!m) continue;
                 if (held + __popc(m) > 32) {   // full: into the list, which lowers the bound

@@ -145,3 +145,34 @@ def test_search_with_the_shortest_wait_limit_ends_and_recovers(C, S):
         for a, b in zip(got, want):
             assert torch.equal(a, b)
     ctx.close()
+
+
+# tiles of 32 candidates up to 256 x 128 of them, of 128 above: both sides of the line, several
+# chunks, ragged last tiles; and every case above through the allocation-free search
+FINE = [("smooth", 1, 256, 128, 3, 8, 1), ("smooth", 1, 331, 99, 3, 8, 1), ("smooth", 3, 257, 128, 3, 8, 1),
+        ("noise", 3, 331, 198, 4, 8, 2), ("noise", 1, 9, 7, 1, 8, 2), ("stripes", 3, 640, 480, 4, 8, 8)]
+
+
+@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", FINE)
+def test_lists_at_the_line_between_tile_sizes(kind, C, W, H, S, leaf, stride):
+    test_seed_lists_equal_the_oracle(kind, C, W, H, S, leaf, stride, 1)
+
+
+@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", CASES + FINE)
+def test_allocation_free_search_equals_the_oracle(kind, C, W, H, S, leaf, stride):
+    import torch
+    f = _frames(kind, C, W, H, W * 1000 + H)
+    f1, f2 = (O.features_all(f[k], S)[0] for k in (0, 1))
+    P = 16 if C == 1 else 32
+    feat = []
+    for x in (f1, f2):
+        y = torch.zeros((H, W, P), dtype=torch.int8, device="cuda")
+        y[..., :9 * C] = torch.from_numpy(np.ascontiguousarray(x).reshape(H, W, 9 * C)).cuda()
+        feat.append(y)
+    ridx, rdist = O.seed_knn(f1, f2, S, leaf, stride)
+    idx = torch.empty(ridx.shape, dtype=torch.int32, device="cuda")
+    dist = torch.empty_like(idx)
+    ff.ff_seed_knn_static(feat[0], feat[1], W, H, C, S, leaf, stride, idx, dist,
+                          torch.cuda.current_stream())
+    np.testing.assert_array_equal(idx.cpu().numpy(), ridx)
+    np.testing.assert_array_equal(dist.cpu().numpy(), rdist)
