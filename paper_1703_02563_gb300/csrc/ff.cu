@@ -1515,14 +1515,11 @@ ff_status ff_features(ff_ctx *c, int slot, const uint8_t *img, int w, int h, int
             int WL, HL;
             level_dims(w, h, L, &WL, &HL);
             uint8_t *out = c->feat[slot] + level_offset(w, h, c->P, L);
-            dim3 grid((WL + 15) / 16, (HL + 15) / 16);
             prof_begin(c, "k_features");
             if (c->C == 1)
-                k_features_tc<1, false><<<grid, tc_feature_threads(L), 0, c->stream>>>(
-                    img, pitch, w, h, L, WL, HL, out, nullptr);
+                launch_features_tc<1, false>(img, pitch, w, h, L, WL, HL, out, nullptr, c->stream);
             else
-                k_features_tc<3, false><<<grid, tc_feature_threads(L), 0, c->stream>>>(
-                    img, pitch, w, h, L, WL, HL, out, nullptr);
+                launch_features_tc<3, false>(img, pitch, w, h, L, WL, HL, out, nullptr, c->stream);
             ff_status s = check_launch(c, "k_features");
             if (s) return s;
         }
@@ -1618,14 +1615,11 @@ ff_status ff_wht_coeffs_tc(const uint8_t *img, int w, int h, int pitch, int chan
     if ((channels != 1 && channels != 3) || level < 0 || level >= FF_MAX_SCALES) return FF_EINVAL;
     int WL, HL;
     level_dims(w, h, level, &WL, &HL);
-    dim3 grid((WL + 15) / 16, (HL + 15) / 16);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (channels == 1)
-        k_features_tc<1, true><<<grid, tc_feature_threads(level), 0, st>>>(
-            img, pitch, w, h, level, WL, HL, nullptr, coeffs_out);
+        launch_features_tc<1, true>(img, pitch, w, h, level, WL, HL, nullptr, coeffs_out, st);
     else
-        k_features_tc<3, true><<<grid, tc_feature_threads(level), 0, st>>>(
-            img, pitch, w, h, level, WL, HL, nullptr, coeffs_out);
+        launch_features_tc<3, true>(img, pitch, w, h, level, WL, HL, nullptr, coeffs_out, st);
     return cudaGetLastError() == cudaSuccess ? FF_OK : FF_ECUDA;
 }
 
@@ -1637,11 +1631,9 @@ ff_status ff_wht_coeffs_scalespace_tc(const uint8_t *img, int w, int h, int pitc
     if (fp16 != 0 && fp16 != 1) return FF_EINVAL;
     int WL, HL;
     level_dims(w, h, level, &WL, &HL);
-    dim3 grid((WL + 15) / 16, (HL + 15) / 16);
     cudaStream_t st = (cudaStream_t)cuda_stream;
 #define FF_LAUNCH_TCS(CC, IN) \
-    k_features_tc<CC, true, IN><<<grid, tc_feature_threads(level), 0, st>>>( \
-        img, pitch, w, h, level, WL, HL, nullptr, coeffs_out)
+    launch_features_tc<CC, true, IN>(img, pitch, w, h, level, WL, HL, nullptr, coeffs_out, st)
     if (channels == 1) {
         if (fp16) FF_LAUNCH_TCS(1, 2);
         else FF_LAUNCH_TCS(1, 1);

@@ -64,19 +64,24 @@ __device__ __forceinline__ void mma_f16_16816(float (&d)[4], const uint32_t (&a)
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Threads of a CTA.  Warps 0-3 do the products; from level 2 on, where a tile's
-// averages sum 16 and more pixels each and a level has few tiles, twelve more help
-// to form them (four levels of a 1242x375 Lab frame: 113 -> 84 us).
-__host__ __device__ constexpr int tc_feature_threads(int L) { return L >= 2 ? 512 : 128; }
+// Whether a CTA has 512 threads instead of 128: on levels of 2 and up, where a tile's
+// averages sum 16 and more pixels each, as long as the level has few tiles; with more of
+// them the GPU is full without the extra warps (128 -> 512 threads, level 2, gray: 240 tiles
+// 10.4 -> 10.3 us, 375 12.3 -> 14.1, 4096 41 -> 83; Lab: 240 tiles 22.6 -> 14.4, 510 25.8 ->
+// 24.6, 920 30.8 -> 43; level 3, Lab: 135 tiles 33 -> 17, 544 41 -> 45).
+constexpr bool tc_feature_wide(int C, int L, long long tiles) {
+    return L >= 2 && tiles <= (C == 3 ? 512 : 256);
+}
 
 // One CTA: a 16x16 tile of level pixels, 4 warps x 4 tile rows; each tile
 // row is one m16 fragment (16 pixels), K = 64 in 4 k-steps of two window
-// rows, N = 9 coefficients padded to 16 (two n8 fragments).
+// rows, N = 9 coefficients padded to 16 (two n8 fragments).  Warps 4 and up (T = 512)
+// only help to form the averages.
 // FLOAT_OUT: write the raw FP32 coefficients [HL][WL][9C] to fout instead
 // of the int8 features.  IN: 0 the rounded integer level image in bf16; 1,
 // 2 the unrounded FP32 scale-space image rounded to bf16, fp16 (FLOAT_OUT).
-template <int C, bool FLOAT_OUT, int IN = 0>
-__global__ void __launch_bounds__(tc_feature_threads(FF_MAX_SCALES))
+template <int C, bool FLOAT_OUT, int IN, int T>
+__global__ void __launch_bounds__(T)
     k_features_tc(const uint8_t *__restrict__ img, int pitch, int W, int H, int L, int WL, int HL,
                   uint8_t *__restrict__ out, float *__restrict__ fout) {
     static_assert(IN == 0 || FLOAT_OUT, "the precision form returns coefficients");
@@ -129,7 +134,7 @@ __global__ void __launch_bounds__(tc_feature_threads(FF_MAX_SCALES))
                                               bf16_sign(wht_basis(k0 + 1, col)));
             }
 #pragma unroll 1
-    for (int rr = 0; rr < 4 && warp < 4; rr++) {
+    for (int rr = 0; rr < 4 && (T == 128 || warp < 4); rr++) {
         const int ty = warp * 4 + rr;
 #pragma unroll
         for (int c = 0; c < C; c++) {
@@ -184,6 +189,18 @@ __global__ void __launch_bounds__(tc_feature_threads(FF_MAX_SCALES))
             reinterpret_cast<uint4 *>(out + ((size_t)y * WL + x) * P)[w] =
                 reinterpret_cast<const uint4 *>(&sOut[p][0])[w];
     }
+}
+
+template <int C, bool FLOAT_OUT, int IN = 0>
+void launch_features_tc(const uint8_t *img, int pitch, int w, int h, int L, int WL, int HL,
+                        uint8_t *out, float *fout, cudaStream_t stream) {
+    const dim3 grid((WL + 15) / 16, (HL + 15) / 16);
+    if (tc_feature_wide(C, L, (long long)grid.x * grid.y))
+        k_features_tc<C, FLOAT_OUT, IN, 512><<<grid, 512, 0, stream>>>(img, pitch, w, h, L, WL, HL,
+                                                                      out, fout);
+    else
+        k_features_tc<C, FLOAT_OUT, IN, 128><<<grid, 128, 0, stream>>>(img, pitch, w, h, L, WL, HL,
+                                                                      out, fout);
 }
 
 }  // namespace ffk

@@ -122,3 +122,20 @@ def test_tc_path_matches_bit_exact():
     np.testing.assert_array_equal(_host(cf), rc)
     np.testing.assert_array_equal(_host(ctx.filter(fwd, bwd)), O.filter_mask(rf, rb, 8))
     ctx.close()
+
+
+# level 2 of 256 and 272 tiles (gray), of 512 and 528 (Lab): the two block sizes of the kernel
+@pytest.mark.parametrize("C,W,H", [(1, 1024, 1024), (1, 1025, 1024), (3, 2048, 1024), (3, 2049, 1024)])
+def test_tensor_core_features_at_the_line_between_block_sizes(C, W, H):
+    import torch
+    f = torch.from_numpy(np.random.default_rng(W).integers(0, 256, (C, H, W), dtype=np.uint8)).cuda()
+    got = []
+    for tc in (0, 1):
+        ctx = ff.Context(ff.Config(channels=C, scales=4, iters=1, max_width=W, max_height=H,
+                                   wht_tensor_cores=tc))
+        ctx.features(0, f)
+        got.append([ctx.features_of(0, L).clone() for L in range(4)])
+        ctx.sync()
+        ctx.close()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
