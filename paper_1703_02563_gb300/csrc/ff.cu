@@ -377,7 +377,8 @@ __global__ void k_rf_init(const uint32_t *__restrict__ flow, const uint8_t *__re
                           int W, int N, int *parent, int *size, uint8_t *flag) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     const bool in = i < N;
-    const bool left = in && lane > 0 && i % W > 0 && rf_joined(flow, mask, i, i - 1);
+    // (the remainder last: masks with few kept points hardly need it)
+    const bool left = in && lane > 0 && rf_joined(flow, mask, i, i - 1) && i % W > 0;
     const unsigned runs = ~__ballot_sync(0xffffffffu, left) & ((2u << lane) - 1u);   // run starts
     if (!in) return;
     parent[i] = mask[i] ? i - (lane - (31 - __clz(runs))) : -1;
@@ -412,6 +413,7 @@ __global__ void k_rf_count(const uint32_t *__restrict__ flow, const uint8_t *__r
         r = rf_find_halve(parent, i);
         atomicMin(parent + i, r);
     }
+    if (!__any_sync(0xffffffffu, kept)) return;
     const unsigned same = __match_any_sync(0xffffffffu, r);
     if (!kept) return;
     if ((int)(threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(size + r, __popc(same));
