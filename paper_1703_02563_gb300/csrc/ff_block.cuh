@@ -107,15 +107,16 @@ __global__ void __launch_bounds__(128)
 constexpr int kBlkCols = 4;                  // columns decided per step
 constexpr int kBlkRows = 4;                  // rows of a strip, one warp each
 constexpr int kBlkCluster = 8;               // strips of a cluster
-// Stager warps: Lab blocks take four (with two a 1024x436 pair 8.19 -> 8.52 ms), gray
-// ones two (with four a 1242x375 pair 5.26 -> 5.55 ms: more of them only contend with
-// the rows for issue slots).
+// Stager warps: Lab blocks take four, gray ones two; more only contend with the rows for
+// issue slots.  One match from seeds, the other number of each (six frame sizes, 128x96 to
+// 1920x1080): Lab with two 6-9% slower (1024x436 3.94 -> 4.23 ms), gray with four 7-10%
+// (1242x375 3.41 -> 3.75 ms).
 __host__ __device__ constexpr int blk_stagers(int C) { return C == 3 ? 4 : 2; }
 __host__ __device__ constexpr int blk_threads(int C) { return (kBlkRows + blk_stagers(C) + 1) * 32; }
 // CTAs per SM that the registers have to allow (0: as they come).  Gray: three, i.e. 80
 // registers; with a few more only two fit, which costs 32 contexts on 640x480 frames
-// 13.3 -> 16.6 ms, and with four, 72 registers, a lone 1242x375 pair takes 3.24 ms
-// instead of 3.00.  Lab: two come (96 registers); three spill (1024x436: 8.4 -> 10.8 ms).
+// 13.3 -> 16.6 ms, and with four, 72 registers, a lone 1242x375 pair takes 8% longer.
+// Lab: two come (96 registers); three spill (1024x436: 8.4 -> 10.8 ms).
 __host__ __device__ constexpr int blk_ctas(int C) { return C == 3 ? 0 : 3; }
 constexpr int kBlkRing = 16;                 // staged blocks per row
 // Levels up to this wide start the next sweep's launch early: its waiting CTAs hold
@@ -383,9 +384,9 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             const uint32_t slot = stage + (uint32_t)(b & (kBlkRing - 1)) * (uint32_t)sizeof(BlockStage);
             // What needs no neighbour: the staged block, the windows of the four columns, the
             // query.  For Lab frames before the wait, where it costs the rows below nothing;
-            // for gray ones, whose evaluations are short, in the shadow of the tap loads
-            // (the 1024x436 Lab pair 8.28 -> 8.00 ms, the 1242x375 gray one 5.81 against
-            // 6.47 ms the other way round).
+            // for gray ones, whose evaluations are short, in the shadow of the tap loads.  (One
+            // match from seeds, the other way round, same six sizes: Lab 1-5% slower, 1024x436
+            // 3.94 -> 4.04 ms; gray 1-6%, 1242x375 3.41 -> 3.61 ms.)
             uint4 cf, cc, ca, cb;
             uint32_t lo1, hi1, lo2, hi2, lo3, hi3;
             int4 seed[LW];
@@ -434,7 +435,15 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             if constexpr (!kEarly) {
                 if (!own_part()) goto finished;
             }
-            const uint4 vf0 = lds128s(vin), vf1 = lds128s(vin + 16);
+            // The four flows above, waited for by other lanes than this one: behind a barrier of the
+            // warp, which a vote is not.  Lab: one here, in the shadow of the tap loads (with the
+            // loads behind the next one 8.43 -> 8.66 ms for the 1024x436 pair).  Gray: the one before
+            // the costs are read (1242x375 pair 2.94 ms; here 3.04).
+            uint4 vf0, vf1;
+            if constexpr (kEarly) {
+                __syncwarp();
+                vf0 = lds128s(vin), vf1 = lds128s(vin + 16);
+            }
             uint32_t acc0 = 0, acc1 = 0;
 #pragma unroll
             for (int k = 0; k < LW; k += 2) {
@@ -449,6 +458,7 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             __syncwarp();
             const uint4 eh = lds128s(cand), ev = lds128s(cand + 16), ra = lds128s(cand + 32),
                         rb = lds128s(cand + 48);
+            if constexpr (!kEarly) vf0 = lds128s(vin), vf1 = lds128s(vin + 16);
             // the better of current and above per column (the latter on ties), with
             // what it would cost at the later columns
             const bool p0 = ev.x <= cc.x, p1 = ev.y <= cc.y, p2 = ev.z <= cc.z, p3 = ev.w <= cc.w;
