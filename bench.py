@@ -400,8 +400,8 @@ def sweep_diagonals(W: int, H: int, cfg) -> int:
 
 
 def step_floor_cycles(peaks: dict) -> float:
-    """Dependent latency of one wavefront step of the sweep, from measured
-    instruction latencies: the row above's decision arrives by a shuffle;
+    """Dependent latency of one step of a sweep that decides one column at a
+    time (the batch sweep's wavefront), from measured instruction latencies: the row above's decision arrives by a shuffle;
     selecting and clamping the candidate (4 ALU), its tap address (9 ALU:
     sign extension, rounding to the level, column and row offsets, 64-bit
     address), one L1-hit load, the byte transpose (2 permutes), one dp4a,
@@ -410,6 +410,32 @@ def step_floor_cycles(peaks: dict) -> float:
     horizontal] into the next step's horizontal source (7 ALU)."""
     return (3 * peaks["lat_shfl"] + peaks["lat_ldg_l1"] + 2 * peaks["lat_prmt"]
             + peaks["lat_dp4a"] + 24 * peaks["lat_alu"])
+
+
+def block_links(W: int, H: int, cfg) -> int:
+    """Links of the serial chain of every block sweep of one direction: a sweep
+    of a U x V level hands its first block of columns down V - 1 rows, and its
+    last row takes ceil(U / 4) blocks."""
+    n = 0
+    for L in range(cfg.scales):
+        wl, hl = level_dims(W, H, L)
+        n += cfg.sweeps(L) * (-(-wl // 4) + hl - 1)
+    return n
+
+
+def block_link_floor_cycles(peaks: dict, channels: int) -> float:
+    """Dependent latency of one link of the block sweep (a row's wait for the
+    block above it to that block's own hand-over), from measured instruction
+    latencies: the poll that sees the flow above (1 shared load) and its vote (1
+    ALU); selecting and clamping the candidate (3 ALU), its tap position and
+    address (8 ALU), one L1-hit load; the byte transpose (2 permutes), one
+    dp4a, the absolute values of one accumulator's words (4 ALU a word; 2 words
+    for Lab, 1 for gray) and their sum over the two lanes (1 shuffle, 3 ALU);
+    the exchange of the costs (1 shared load); and the four columns' compares
+    and selects into the flow that is handed on (14 ALU)."""
+    alu = 1 + 3 + 8 + 4 * (2 if channels == 3 else 1) + 3 + 14
+    return (2 * peaks["lat_lds"] + peaks["lat_ldg_l1"] + 2 * peaks["lat_prmt"] + peaks["lat_dp4a"]
+            + peaks["lat_shfl"] + alu * peaks["lat_alu"])
 
 
 # ----------------------------------------------------------------------------
@@ -552,15 +578,17 @@ def roofline(res: dict, steps: int, n_dirs: int) -> dict:
     """Roofline of the kernel with the largest share of device time.
 
     k_sweep (propagation + random search) is integer-ALU work on a serial
-    wavefront.  Its algorithmic work is OPS_PER_DIM integer operations per
+    chain.  Its algorithmic work is OPS_PER_DIM integer operations per
     feature dimension per evaluation (evaluations per launch from
     sweep_evals); the peak is the same arithmetic's measured throughput
     (ff_measure_peaks: sad_dims_per_s x OPS_PER_DIM), with the dp4a
     instruction peak (8 ops per dp4a) beside it.  Its L2 fraction is the L2
     traffic of one launch (ncu record) over the launch time, against the
-    measured L2 read bandwidth.  Its critical path is the cycles per
-    anti-diagonal (device time x SM clock over the sweeps' anti-diagonals)
-    against the dependent latency of one step (step_floor_cycles).
+    measured L2 read bandwidth.  What bounds it is block_path: the cycles per
+    link of the block sweep's chain (device time x SM clock over the links,
+    block_links) against a link's dependent latency (block_link_floor_cycles).
+    critical_path divides the same time by the anti-diagonals of a sweep of one
+    column per step, for comparison: the block sweep has fewer links than that.
     k_seed_scan (the tensor-core seeding) is a dense contraction: 2 flops per
     multiply-add of (queries x candidates x K), against the measured bf16
     tensor peak.
@@ -600,6 +628,15 @@ def roofline(res: dict, steps: int, n_dirs: int) -> dict:
         diags = n_dirs * steps * sweep_diagonals(W, H, res["cfg"])
         cyc = ms / 1e3 * clk * 1e6 / diags
         floor = step_floor_cycles(peaks)
+        block = None
+        if "lat_lds" in peaks:
+            link = ms / 1e3 * clk * 1e6 / (n_dirs * steps * block_links(W, H, res["cfg"]))
+            link_floor = block_link_floor_cycles(peaks, C)
+            block = {"cycles_per_link": link, "floor_cycles": link_floor,
+                     "frac": link_floor / link, "sm_mhz": clk,
+                     "links": "V_L - 1 row hand-overs and ceil(U_L / 4) blocks of every sweep",
+                     "floor": "dependent latency of one link from measured instruction "
+                              "latencies (block_link_floor_cycles)"}
         return {"kernel": dom, "bound": "alu", "achieved": achieved, "peak": peak,
                 "unit": "Tops/s", "frac": achieved / peak, "traffic": traffic,
                 "launches": n_launch, "avg_launch_ms": avg_ms, "share": share, "timing": timing,
@@ -608,18 +645,21 @@ def roofline(res: dict, steps: int, n_dirs: int) -> dict:
                 "peak_source": "measured (ff_measure_peaks): the matching error's per-dimension "
                                f"arithmetic at full occupancy, {OPS_PER_DIM} ops per dimension",
                 "dp4a_peak": dp4a_peak, "frac_of_dp4a_peak": achieved / dp4a_peak,
-                "l2": l2,
+                "l2": l2, "block_path": block,
                 "critical_path": {"cycles_per_step": cyc, "floor_cycles": floor,
                                   "frac": floor / cyc, "sm_mhz": clk,
-                                  "steps": "anti-diagonals U_L + V_L - 1 of every sweep",
-                                  "floor": "dependent latency of one step from measured "
+                                  "steps": "anti-diagonals U_L + V_L - 1 of every sweep, of a "
+                                           "sweep of one column per step (the kernel's own "
+                                           "chain: block_path)",
+                                  "floor": "dependent latency of one such step from measured "
                                            "instruction latencies (step_floor_cycles)"}}
     if dom == "k_seed_scan":
         N = 1 << (S - 1)
         nq = ((W + N - 1) // N) * ((H + N - 1) // N)
         K = 16 if C == 1 else 32
-        ncand = ((W + 1) // 2) * ((H + 1) // 2) if res["cfg"].seed_stride == 2 else W * H
-        flops = n_dirs * steps * 2 * nq * ncand * K * 2 * (1 + 1 / 16) / max(n_launch, 1)
+        st = res["cfg"].seed_stride
+        ncand = -(-W // st) * -(-H // st)
+        flops = n_dirs * steps * nq * ncand * K * 2 / max(n_launch, 1)
         peak = measured_peaks().get("bf16_tflops", 1900.0)
         achieved = flops / (avg_ms / 1e3) / 1e12
         return {"kernel": dom, "bound": "tensor", "achieved": achieved, "peak": peak,

@@ -79,6 +79,27 @@ def test_sweep_roofline_arithmetic():
     assert "timed region" in r2["timing"] and "profiled pass" in r["timing"]
 
 
+def test_block_sweep_path_and_search_rate():
+    cfg = ff.Config(channels=3, scales=2, iters=5, seed_stride=3)
+    W, H = 65, 48
+    peaks = {"sad_dims_per_s": 5e12, "dp4a_per_s": 2e13, "l2_read_gbs": 2e4, "lat_lds": 30.0,
+             "lat_shfl": 20.0, "lat_ldg_l1": 40.0, "lat_prmt": 5.0, "lat_dp4a": 6.0,
+             "lat_alu": 4.0}
+    res = {"kstats": {"k_sweep": (10, 20.0), "k_features": (2, 0.5)},
+           "W": W, "H": H, "C": 3, "S": 2, "I": 5, "cfg": cfg, "workload": "none",
+           "peaks": peaks, "clocks": {"sm_mhz": 2000.0}}
+    # by hand: level 0 65x48 (17 blocks), level 1 33x24 (9 blocks); 5 sweeps each
+    links = 5 * (17 + 47) + 5 * (9 + 23)
+    b = bench.roofline(res, steps=1, n_dirs=1)["block_path"]
+    assert b["cycles_per_link"] == pytest.approx(20.0e-3 * 2000e6 / links)
+    assert b["floor_cycles"] == pytest.approx(2 * 30 + 40 + 2 * 5 + 6 + 20 + 37 * 4)
+    assert b["frac"] == pytest.approx(b["floor_cycles"] / b["cycles_per_link"])
+    # the search: one product of every query with every third pixel, K = 32, per direction
+    res["kstats"] = {"k_seed_scan": (4, 8.0)}
+    r = bench.roofline(res, steps=2, n_dirs=2)
+    assert r["achieved"] == pytest.approx(33 * 24 * 22 * 16 * 32 * 2 / 2e-3 / 1e12)
+
+
 def test_code_hash_ignores_comments_not_code(tmp_path, monkeypatch):
     # the recorded ncu counters stay valid across comment edits only
     monkeypatch.setattr(bench, "ROOT", str(tmp_path))
