@@ -235,8 +235,8 @@ ff_status ff_seed_knn(ff_ctx *ctx, ff_dir dir, int32_t *idx_out, int32_t *dist_o
  * hands libraries a fixed budget, or a real-time loop that must never wait
  * on the allocator (cudaMalloc and cudaFree can synchronise the device and
  * stall every stream).  It computes what ff_seed_knn computes, without a
- * context, and allocates nothing: its scratch (the per-chunk partial lists)
- * is an 8 MiB array in the library's static device memory, which every GPU
+ * context, and allocates nothing: its scratch (each chunk's lists of tiles) is
+ * an 8 MiB array in the library's static device memory, which every GPU
  * that loads the library holds until the process exits.
  *  feat_src0 / feat_dst0: level-0 features of the query and the candidate
  *    frame, int8 [h][w][P] (P = 16 for 1 channel, 32 for 3: the 9*channels
@@ -291,9 +291,12 @@ ff_status ff_sync(ff_ctx *ctx);
  * FF_DEBUG_SWEEP_LANES: which sweep kernel runs, 4 (default; 8 means the same:
  * blocks of four columns, a warp per row, the shortest time for one pair) or 2
  * (two lanes of a warp per grid point, 16 rows per strip: fewer instructions
- * per point; what batch and server slots run).  FF_DEBUG_SEED_TC: accepted; the
- * seeding search has one path, on the tcgen05 tensor cores.  Every value gives
- * the same results. */
+ * per point; what batch and server slots run).  A program that keeps many
+ * contexts busy at once, on a stream each, fills the GPU with either and gets
+ * more out of 2: matches from seeds at 1024x436 Lab take 3.9 ms (8.2 with 2)
+ * with 4 contexts, 11.9 (10.9) with 16 and 23.1 (15.8) with 32.
+ * FF_DEBUG_SEED_TC: accepted; the seeding search has one path, on the tcgen05
+ * tensor cores.  Every value gives the same results. */
 typedef enum {
     FF_DEBUG_WAIT_LIMIT_NS = 1,
     FF_DEBUG_FORCE_TIMEOUT = 2,
@@ -312,10 +315,12 @@ ff_status ff_debug_set(ff_ctx *ctx, ff_debug_key key, long long value);
  * mode) clears the record and starts recording; ff_profile(ctx, 0) stops (an
  * open run ends there).  Any other mode: FF_EINVAL.  ff_kernel_stats (call
  * after ff_sync) returns, for the kernel named `kernel` ("k_features",
- * "k_seed_prep", "k_seed_scan", "k_seed_merge", "k_seed_rerank",
- * "k_seed_given", "k_upsample", "k_sweep", "k_export", "k_filter", "k_dense",
- * "k_region", "k_sparsify"), the number of recorded launches and their summed
- * device time in milliseconds. */
+ * "k_seed_prep", "k_seed_scan", "k_seed_merge" (the ranking and, for a match,
+ * the coarsest costs), "k_seed_given", "k_upsample", "k_sweep", "k_search"
+ * (the random search where no sweep follows to do it), "k_export",
+ * "k_filter", "k_dense", "k_region", "k_sparsify"; "k_seed_rerank" is accepted
+ * and has no launches of its own), the number of recorded launches and their
+ * summed device time in milliseconds. */
 typedef enum { FF_PROFILE_LAUNCHES = 1, FF_PROFILE_SWEEP_RUNS = 2 } ff_profile_mode;
 ff_status ff_profile(ff_ctx *ctx, int mode);
 ff_status ff_kernel_stats(ff_ctx *ctx, const char *kernel, long long *launches,

@@ -1299,8 +1299,8 @@ ff_status region_into(ff_ctx *c, const int16_t *fwd, const uint8_t *mask_in, int
 // ============================================================================
 namespace {
 
-// Scratch of the allocation-free seeding search: the per-chunk partial top-8
-// lists, 8 MiB.  It lives in this file's static device memory, so every GPU
+// Scratch of the allocation-free seeding search: every query's lists of tiles, one of
+// eight words per chunk (kTcTileBits), 8 MiB.  It lives in this file's static device memory, so every GPU
 // that loads the library holds it until the process exits.  Every call
 // shares it; calls that overlap on a GPU race on it.
 constexpr size_t kStaticScratchInt2 = (size_t)1 << 20;   // 8 MiB of int2
@@ -1769,7 +1769,7 @@ ff_status ff_seed_knn_static(const int8_t *feat_src0, const int8_t *feat_dst0, i
     int WS, HS;
     level_dims(w, h, scales - 1, &WS, &HS);
     const size_t nq = (size_t)WS * HS;
-    const size_t max_slots = kStaticScratchInt2 / 8;   // (chunk, query) lists that fit
+    const size_t max_slots = kStaticScratchInt2 / 8;   // the lists of two chunks then fit
     if (nq > max_slots)
         return *msg = "too many coarsest-grid points for the static scratch (limit 131072)",
                FF_EINVAL;

@@ -137,11 +137,7 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
     return v;
 }
 
-__device__ __forceinline__ void st_relaxed_u64(unsigned long long *p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// the same, under a predicate (no branch around the store)
+// a relaxed store under a predicate (no branch around it)
 __device__ __forceinline__ void st_relaxed_u64_if(unsigned long long *p, unsigned long long v,
                                                   bool pred) {
     asm volatile(
@@ -154,20 +150,6 @@ __device__ __forceinline__ int ld_relaxed_i32(const int *p) {
     int v;
     asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-
-// named barrier 1 over `n` threads with an OR-reduction of `pred`
-__device__ __forceinline__ int bar_or(int pred, int n) {
-    int out;
-    asm volatile(
-        "{\n\t.reg .pred pi, po;\n\t"
-        "setp.ne.s32 pi, %1, 0;\n\t"
-        "bar.red.or.pred po, 1, %2, pi;\n\t"
-        "selp.s32 %0, 1, 0, po;\n\t}"
-        : "=r"(out)
-        : "r"(pred), "r"(n)
-        : "memory");
-    return out;
 }
 
 }  // namespace ffk
