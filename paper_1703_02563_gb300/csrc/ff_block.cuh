@@ -203,11 +203,6 @@ __device__ __forceinline__ unsigned long long lds64s(uint32_t p) {
     asm volatile("ld.volatile.shared.b64 %0, [%1];" : "=l"(v) : "r"(p) : "memory");
     return v;
 }
-__device__ __forceinline__ uint32_t lds32s(uint32_t p) {
-    uint32_t v;
-    asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(v) : "r"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ uint4 lds128s(uint32_t p) {
     uint4 r;
     asm volatile("ld.volatile.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
@@ -497,7 +492,8 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             const uint32_t c0 = min(eh.x, bc0), c1 = min(e1, bc1), c2 = min(e2, bc2), c3 = min(e3, bc3);
             const uint32_t dc = j < 2 ? (j == 0 ? c0 : c1) : (j == 2 ? c2 : c3);
             stg_u32_if(state_row, lane < 4 ? df : dc, lane < 8 && inside);
-            if (lane == 0) sts32s(done, b + 1);
+            // (every lane has read the staged block: they met before the costs were read)
+            if (lane == 0) sts32_release(done, (uint32_t)(b + 1));
             out += 8 * kBlkCols;
             vin += 8 * kBlkCols;
             edge += kBlkCols;
@@ -522,10 +518,11 @@ __global__ void __cluster_dims__(kBlkCluster, 1, 1)
             for (int k = 1;; k++) {
                 if (k > 1) __nanosleep(200);
                 const bool ok = lane >= kBlkRows ||
-                                (int)lds32s(smem_addr(&sm.done[lane])) + kBlkRing >= 2 * p + 2;
+                                (int)lds32_acquire(smem_addr(&sm.done[lane])) + kBlkRing >= 2 * p + 2;
                 if (__all_sync(FULL, ok)) break;
                 if (wait_over(k, t0, a.wait_ns, v_abort, a.err)) goto finished;
             }
+            __syncwarp();          // (four lanes have looked, all will write)
             if (p == 0) launch_dependents();   // (the next sweep's launch may come in)
             const int u = 8 * p + (lane & 7);
             const bool in = v < V && u < U;
