@@ -565,6 +565,10 @@ __global__ void __launch_bounds__(128)
     for (int k = 0; k < 8; k += FINE ? 4 : 1) {
         const int t = __shfl_sync(FULL, best.I, k);
         if (t == 0x7fffffff) break;
+        if (bI != 0x7fffffff) {    // eight are known: may this tile, or one behind it, hold a better one?
+            const int c = t * trows, cy = c / Wc, first = (cy * W + (c - cy * Wc)) * stride;
+            if (!lex_less(__shfl_sync(FULL, best.D, k) - kTcKeyBias + qn, first, bD, bI)) break;
+        }
         const int end = FINE ? t * trows + 1 : min((t + 1) * trows, ncand);
         for (int o0 = t * trows; o0 < end; o0 += kTcRows) {
             uint4 r[4][NV];

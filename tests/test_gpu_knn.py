@@ -158,7 +158,18 @@ def test_lists_at_the_line_between_tile_sizes(kind, C, W, H, S, leaf, stride):
     test_seed_lists_equal_the_oracle(kind, C, W, H, S, leaf, stride, 1)
 
 
-@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", CASES + FINE)
+# equal candidates, where the ranking ends at the first tile that cannot hold a better one: tiles
+# of 32 and of 128, strides, two halves of one vector each
+TIES = [("constant", 3, 331, 99, 2, 8, 4), ("constant", 1, 331, 199, 3, 5, 1), ("stripes", 1, 331, 99, 2, 8, 3),
+        ("stripes", 3, 333, 201, 4, 7, 1)]
+
+
+@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", TIES)
+def test_lists_of_equal_candidates(kind, C, W, H, S, leaf, stride):
+    test_seed_lists_equal_the_oracle(kind, C, W, H, S, leaf, stride, 1)
+
+
+@pytest.mark.parametrize("kind,C,W,H,S,leaf,stride", CASES + FINE + TIES)
 def test_allocation_free_search_equals_the_oracle(kind, C, W, H, S, leaf, stride):
     import torch
     f = _frames(kind, C, W, H, W * 1000 + H)
