@@ -282,7 +282,7 @@ __device__ __forceinline__ bool wait_over(int k, unsigned long long &t0, unsigne
 // What bounds it: a step of ~1060 cycles (U/4 of them) and a row hand-over of ~870
 // (V of them), both chains of dependent instructions of one warp (about 5 cycles
 // each) with one tap load in them; 57% of the time are the hand-overs.  At 1024x436
-// Lab the level-0 sweep takes 406 us (650 with a step of one column of eight rows,
+// Lab the level-0 sweep takes 373 us with cold caches (650 with a step of one column of eight rows,
 // ~920 cycles on each of U + V anti-diagonals).  Two columns per step would double
 // the steps for about a tenth less of a hand-over; eight need 44 costs per step.
 // Four rows per strip keep one row warp on each quarter of an SM.

@@ -565,7 +565,9 @@ __global__ void __launch_bounds__(128)
     for (int k = 0; k < 8; k += FINE ? 4 : 1) {
         const int t = __shfl_sync(FULL, best.I, k);
         if (t == 0x7fffffff) break;
-        if (bI != 0x7fffffff) {    // eight are known: may this tile, or one behind it, hold a better one?
+        // eight are known: may this tile, or one behind it, hold a better one?  (Uniform frames,
+        // 76800 queries, Lab: the search 195 -> 147 us with every eighth pixel; others unchanged.)
+        if (bI != 0x7fffffff) {
             const int c = t * trows, cy = c / Wc, first = (cy * W + (c - cy * Wc)) * stride;
             if (!lex_less(__shfl_sync(FULL, best.D, k) - kTcKeyBias + qn, first, bD, bI)) break;
         }
